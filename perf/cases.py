@@ -33,7 +33,7 @@ def listed():
     return [
         # a small graph, one call: an interactive query, bound by launches and host work
         {"name": "triangle_uniform_4k", "kind": "join", "query": "triangle", "graph": "uniform", "scale": 12, "ef": 8,
-         "cells": "1,1,1", "mode": "count"},
+         "cells": "1,1,1", "mode": "count", "tuned": False},
         # a service's burst of requests, each with a selection of its own, over three resident graphs
         {"name": "serve_rmat20_burst48", "kind": "serve", "scale": 20, "requests": 48, "sample": 16384},
         # an analyst's many small graphs: one replayed launch for 96 triangle and 4-clique counts
@@ -44,20 +44,20 @@ def listed():
         # loading a relation whose ids are 32-bit hashes, by its second attribute, a ragged size
         {"name": "build_hashed_3m", "kind": "build", "graph": "uniform", "scale": 18, "ef": 12, "ids": "hashed",
          "order": 1, "drop": 40007},
-        # the benchmark's query in the benchmark's 64 cells, counted per cell: the largest search
+        # the benchmark's query in the benchmark's 64 cells with its tuned schedule, counted per cell: the largest search
         {"name": "triangle_rmat22_64cells", "kind": "join", "query": "triangle", "graph": "rmat", "scale": 22,
-         "ef": 16, "cells": "64,1,1", "mode": "count"},
-        # all triangles of a mid-size graph written out in a fixed order, both attributes partitioned
+         "ef": 16, "cells": "64,1,1", "mode": "count", "tuned": True},
+        # all triangles of a mid-size graph written out in a fixed order, the tuned schedule, both attributes partitioned
         {"name": "triangle_rmat19_tuples", "kind": "join", "query": "triangle", "graph": "rmat", "scale": 19,
-         "ef": 16, "cells": "4,4,1", "mode": "materialize"},
+         "ef": 16, "cells": "4,4,1", "mode": "materialize", "tuned": True},
         # a materialized view: the triangles in one pass, then indexed for the next query
         {"name": "view_rmat17", "kind": "view", "scale": 17, "ef": 16},
         # the deep query of the benchmark, with its intersections rewritten
         {"name": "clique4_rmat17", "kind": "join", "query": "clique4", "graph": "rmat", "scale": 17, "ef": 16,
-         "cells": "1,1,1,1", "mode": "count"},
+         "cells": "1,1,1,1", "mode": "count", "tuned": False},
         # closed 4-walks of a symmetric graph: the longest search for its rows
         {"name": "cycle4_rmat13", "kind": "join", "query": "cycle4", "graph": "rmat", "scale": 13, "ef": 16,
-         "cells": "1,1,1,1", "mode": "count"},
+         "cells": "1,1,1,1", "mode": "count", "tuned": False},
         # Loomis-Whitney on resident dense tensors
         {"name": "lw_dense_256", "kind": "tensor", "n": 256, "fill": "dense", "spread": 1, "cells": "1,1,1,1",
          "load": False},
@@ -84,11 +84,12 @@ def draw(rng):
         low, top = {"triangle": (8, 20), "cycle4": (8, 12), "diamond": (8, 12), "clique4": (8, 16),
                     "two_triangle": (8, 10)}[q]
         nv = QUERIES[q].n_vars
+        mode = rng.choice(["count", "count", "materialize"]) if q == "triangle" else "count"
         cells = rng.choice([[1] * nv, [1] * nv, [rng.choice([3, 16, 64])] + [1] * (nv - 1),
                             [rng.choice([2, 4]), rng.choice([2, 5])] + [1] * (nv - 2)])
         return {"kind": kind, "query": q, "graph": graph, "scale": rng.randint(low, top),
                 "ef": rng.randint(8, 16) if q != "two_triangle" else 8, "cells": ",".join(map(str, cells)),
-                "mode": rng.choice(["count", "count", "materialize"]) if q == "triangle" else "count"}
+                "mode": mode, "tuned": mode == "materialize" or rng.random() < 0.3}
     if kind == "view":
         return {"kind": kind, "scale": rng.randint(9, 17), "ef": rng.randint(4, 16)}
     if kind == "serve":
@@ -105,6 +106,10 @@ def draw(rng):
 
 
 # ------------------------------------------------------------------- inputs
+
+# the schedule the benchmark's autotuner settles on: short work items, no merge path
+TUNED = {"item_grain": 16, "merge_min": 0xFFFFFFFF, "merge_ratio": 1}
+
 
 def _gen(seed):
     return torch.Generator(device=DEV).manual_seed(seed & 0x7FFFFFFFFFFFFFFF)
@@ -290,7 +295,7 @@ def run(st):
     if kind == "join":
         many = max(_cells(case)) > 1
         r = hc.run_join(st["query"], st["indexes"], shares=_cells(case), mode=case["mode"], cell_counts=many,
-                        keep_device=True)
+                        keep_device=True, **(TUNED if case["tuned"] else {}))
         out = {"count": r.count}
         if many:
             out["cells"] = r.cell_counts
