@@ -399,6 +399,36 @@ __device__ __forceinline__ bool dir_find(P a, const uint4* __restrict__ g, uint3
     return dir_walk_find(a, dir_load(g, (uint64_t)lo + k), hi, x, pos);
 }
 
+// ------------------------------------------------------------ dense bitmaps
+// Runs that hold about one in eight of the values they span, or more, are
+// also kept as bitmaps, at 8 bits a value of the level: a run a[lo, hi) of
+// n >= DIR_MIN values owns the 32-bit words that lie wholly in bytes [lo, hi)
+// of an array (so runs share no word), and is dense when its values fit
+// there: with vbase = vmin rounded down to a multiple of 32, bit b of its
+// word w stands for the value vbase + 32 w + b.  A dense run is searched by
+// one bit, and two of them intersect word by word.  The array starts with a
+// header of DENSE_HEAD words, the first of which is nonzero when any run is
+// dense (a large sparse graph has none, and its searches skip all this).
+constexpr uint32_t DENSE_HEAD = 4;
+
+struct Dense {
+    uint32_t w0;     // the run's first word, in the array with its header
+    uint32_t vbase;  // value of bit 0
+    uint32_t span;   // vmax - vbase: values above it are absent
+    bool ok;         // the run is dense
+};
+
+// n = hi - lo >= DIR_MIN, so the run has at least 3 whole words.
+__device__ __forceinline__ Dense dense_of(uint32_t lo, uint32_t hi, uint32_t vmin, uint32_t vmax) {
+    Dense D;
+    const uint32_t w = (uint32_t)(((uint64_t)lo + 3u) >> 2);
+    D.w0 = w + DENSE_HEAD;
+    D.vbase = vmin & ~31u;
+    D.span = vmax - D.vbase;
+    D.ok = vmax >= vmin && (D.span >> 5) < (hi >> 2) - w;
+    return D;
+}
+
 #endif  // __CUDACC__
 
 // --------------------------------------------------------------- host entry
@@ -417,9 +447,11 @@ hc_status build_unary_impl(const uint32_t* d_values, uint64_t n, uint32_t max_va
 // Bucket directory g (parallel to a, alen 16-byte entries, allocated here) of the
 // runs [o[r], o[r+1]) of a, r < nruns (nruns = min(nruns_max, *d_nruns) when
 // d_nruns is given), or with o == NULL of the one run [0, nruns_max);
-// nothing is computed once *d_err is set.
+// nothing is computed once *d_err is set.  out_b receives the bitmaps of
+// the dense runs (dense_of) likewise (none are built when it is NULL).
 hc_status build_directory(const uint32_t* a, uint64_t alen, const uint32_t* o, uint64_t nruns_max,
-                          const uint32_t* d_nruns, const uint32_t* d_err, cudaStream_t s, uint4** out_g);
+                          const uint32_t* d_nruns, const uint32_t* d_err, cudaStream_t s, uint4** out_g,
+                          uint32_t** out_b);
 
 // Device-wide exclusive scan of counts into uint64 offsets; out[n] receives
 // the total.  n = min(n_max, *d_n) when d_n is given (a device-side count),

@@ -326,3 +326,29 @@ def test_dense_runs(hc, pair_min):
     c32 = np.array(list(itertools.product(range(3), range(3), range(32))), dtype=np.uint32)
     run_both(hc, 4, LW_ATOMS, [c32, c32, c32, c32], pair_min=pair_min)
     run_both(hc, 4, CT_ATOMS, [cube, holes, cube], pair_min=pair_min)
+
+
+@pytest.mark.parametrize("base", [0, 31, 1000, 0xFFFFFFFF])
+@pytest.mark.parametrize("n", [15, 16, 33, 700])
+def test_dense_bitmaps(hc, n, base):
+    """Last-loop lists around the limits of the dense-run bitmaps: runs of 15
+    (no directory) and 16 values, spans just inside and outside 8 bits a
+    value, starts at and off a word's edge, a list ending at 0xFFFFFFFF, and
+    lists of which only some are dense, counted and materialized."""
+    rng = np.random.default_rng(n)
+    sets = []
+    for span in (n, n + 33, 8 * n - 70, 8 * n - 31, 8 * n + 1, 12 * n):
+        span = max(span, n)
+        v = np.sort(rng.choice(span, size=n, replace=False)).astype(np.uint64)
+        v[0], v[-1] = 0, span - 1
+        v = np.unique(v)
+        lo = base if base != 0xFFFFFFFF else base - (span - 1)
+        sets.append((v + np.uint64(lo)).astype(np.uint32))
+    r = np.concatenate([np.stack([np.full(s.shape[0], i, np.uint32), s], axis=1) for i, s in enumerate(sets)])
+    t = np.array(list(itertools.product(range(len(sets)), repeat=2)), dtype=np.uint32)
+    # Q(x, y, u) <- R(x, u), R(y, u), T(x, y); and with a third list S(u) of every second value
+    run_both(hc, 3, [(0, 2), (1, 2), (0, 1)], [r, r, t])
+    s = np.unique(r[:, 1])[::2].reshape(-1, 1).copy()
+    run_both(hc, 3, [(0, 2), (1, 2), (0, 1), (2,)], [r, r, t, s])
+    # the last loop is the second: its list is cut into work items
+    run_both(hc, 2, [(0, 1), (1,)], [r, s], item_grain=7)
