@@ -291,7 +291,8 @@ typedef struct {
     uint32_t merge_min;           /* last loop: two lists both at least this long ...   */
     uint32_t merge_ratio;         /* ... and within this length ratio are intersected    */
                                   /* by a warp block merge, others by binary search      */
-                                  /* (0: defaults 32 and 4; 0xFFFFFFFF: never merge)     */
+                                  /* (0: 32 and 4; 0xFFFFFFFF: never merge; with both 0   */
+                                  /* only where the longer list has no directory)        */
     uint32_t slice_grain;         /* 4+ loops: loop-3 candidates per work slice of a     */
                                   /* loop-2 binding (0: default 256; 0xFFFFFFFF: none)   */
     uint32_t lift_arena;          /* query rewriting: words of device scratch per warp   */
