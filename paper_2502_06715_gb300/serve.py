@@ -50,8 +50,14 @@ class Outcome:
 def _selection_values(values) -> np.ndarray:
     """A request's selection as the unary builder needs it: uint32 values,
     strictly ascending (sorted and de-duplicated on the host, because the
-    builder trusts its input order and takes the last value as the largest)."""
-    return np.unique(np.asarray(values, dtype=np.uint32))
+    builder trusts its input order and takes the last value as the largest).
+    A sort and a comparison of neighbours: numpy's unique hashes first, and at
+    16,384 values took 1.5 of a request's 2.0 ms of host time."""
+    v = np.sort(np.asarray(values, dtype=np.uint32), axis=None)
+    distinct = np.empty(v.shape, dtype=bool)
+    distinct[:1] = True
+    np.not_equal(v[1:], v[:-1], out=distinct[1:])
+    return v if distinct.all() else v[distinct]
 
 
 def _unary_index(values: np.ndarray | None, device, stream) -> Index | None:
