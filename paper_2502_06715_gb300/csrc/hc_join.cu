@@ -139,42 +139,67 @@ __global__ void l0_count_kernel(const DPlan* __restrict__ gP, uint32_t* __restri
     }
 }
 
-// Candidate t -> (cell, value of the cell's shortest loop-1 list); probe the
-// other loop-1 lists.  WRITE=false stores the match flag (0 past the last
-// candidate); WRITE=true writes each matching candidate as an entry at its
-// compacted slot, with the ranges of the atoms it opens and its number of
-// loop-2 candidates.
-// Nothing runs once the join's error word is set (a scan before it gave up
-// a wait, so its offsets are not valid).
-template <bool WRITE>
-__global__ void l0_probe_kernel(const DPlan* __restrict__ gP, const uint64_t* __restrict__ candoff, uint64_t tmax,
-                                uint32_t* __restrict__ flags, const uint64_t* __restrict__ flagoff,
-                                uint32_t* __restrict__ e_cell, uint32_t* __restrict__ e_x,
-                                uint32_t* __restrict__ e_rng, uint64_t* __restrict__ e_units,
-                                uint32_t* __restrict__ e_split, const JoinCtl* __restrict__ ctl) {
-    __shared__ DPlan P;
-    load_plan(P, gP);
-    if (dev_err_set(&ctl->err)) return;
-    const uint64_t T = min(tmax, candoff[P.ncells]);
+// One query's loop-1 pass: where its candidates come from and where its
+// entries go.
+struct L0Job {
+    const DPlan* plan;        // device copy of the plan (l0_kernel writes it, l0_batch_kernel reads it)
+    const uint64_t* candoff;  // prefix of the cells' candidate counts, or NULL with one cell
+    uint64_t ncand;           // candidates, at most (exactly, with one cell)
+    uint32_t *e_cell, *e_x, *e_rng, *e_split;
+    uint64_t* uoff;
+    JoinCtl* ctl;
+    uint64_t* status;  // look-back words: [tiles] entry counts, then [tiles] work units
+    uint32_t tiles;
+    uint32_t tile0;  // batched: the query's first tile
+};
+
+// A tile of loop 1: thread t's candidate is value t of the concatenation of
+// the cells' shortest loop-1 lists, searched in the cell's other loop-1 lists.
+// A match becomes an entry: its cell, value, the ranges of the atoms it opens
+// and its work units (loop-2 candidates, each cut into slices of its loop-3
+// candidates when the entry fixes a long loop-3 list).  Entries keep the
+// candidates' order: the tile's matches and units are scanned, and the tile's
+// offsets come from two decoupled look-backs, one warp each.  The tile that
+// holds the last candidate closes uoff and n_entries.  All threads call;
+// false when this tile and those after it hold no candidate.
+constexpr uint32_t L0_TILE = 256;
+constexpr uint32_t L0_WARPS = L0_TILE / 32;
+struct L0Shared {
+    uint32_t wcnt[L0_WARPS];
+    uint64_t wunits[L0_WARPS];
+    uint64_t excl[2];
+    uint64_t ncand;
+};
+
+__device__ __forceinline__ bool l0_tile(const DPlan& P, const L0Job& J, uint32_t tile, uint64_t wait_ns, L0Shared& sh) {
+    const uint32_t tid = threadIdx.x, lane = lane_id(), w = tid >> 5;
+    // nothing runs once the join's error word is set (a scan before it gave up
+    // a wait, so its offsets are not valid); read once for the whole block
+    if (tid == 0)
+        sh.ncand = dev_err_set(&J.ctl->err) ? 0 : J.candoff ? min(J.ncand, J.candoff[P.ncells]) : J.ncand;
+    __syncthreads();
+    const uint64_t T = sh.ncand;
+    const uint64_t base = (uint64_t)tile * L0_TILE;
+    if (tile > 0 && base >= T) return false;  // no tile with candidates waits on this one
+    const uint64_t t = base + tid;
     const int n0 = P.nsrc[0];
-    const uint64_t tend = WRITE ? T : tmax;
-    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < tend; t += (uint64_t)gridDim.x * blockDim.x) {
-        if (!WRITE && t >= T) {
-            flags[t] = 0;
-            continue;
+    bool ok = t < T;
+    uint32_t c = 0, x = 0, split = 1, m = 0;
+    uint32_t rlo[MAXOPEN], rhi[MAXOPEN], pos[MAXOPEN];
+    if (ok) {
+        uint32_t k = (uint32_t)t;
+        if (J.candoff != nullptr) {
+            uint32_t lo = 0, hi = P.ncells;  // last cell c with candoff[c] <= t
+            while (hi - lo > 1) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (J.candoff[mid] <= t)
+                    lo = mid;
+                else
+                    hi = mid;
+            }
+            c = lo;
+            k = (uint32_t)(t - J.candoff[c]);
         }
-        if (WRITE && flags[t] == 0) continue;
-        uint32_t lo = 0, hi = P.ncells;  // last cell c with candoff[c] <= t
-        while (hi - lo > 1) {
-            uint32_t mid = (lo + hi) >> 1;
-            if (candoff[mid] <= t)
-                lo = mid;
-            else
-                hi = mid;
-        }
-        const uint32_t c = lo;
-        const uint32_t k = (uint32_t)(t - candoff[c]);
-        uint32_t rlo[MAXOPEN], rhi[MAXOPEN];
         uint32_t best = 0, bestlen = 0xFFFFFFFFu;
 #pragma unroll
         for (int q = 0; q < MAXOPEN; ++q) {
@@ -187,50 +212,39 @@ __global__ void l0_probe_kernel(const DPlan* __restrict__ gP, const uint64_t* __
                 }
             }
         }
-        uint32_t x = 0;
 #pragma unroll
         for (int q = 0; q < MAXOPEN; ++q)
             if (q == (int)best) x = P.atom[P.src_atom[0][q]].v1[rlo[q] + k];
-        bool ok = true;
-        uint32_t pos[MAXOPEN];
 #pragma unroll
         for (int q = 0; q < MAXOPEN; ++q) {
             pos[q] = 0;
-            if (q < n0) {
+            if (q < n0 && ok) {
                 const DAtom& a = P.atom[P.src_atom[0][q]];
                 uint32_t p;
                 if (q == (int)best) {
                     p = rlo[q] + k;
                 } else if (a.v1pos != nullptr) {  // direct position of x in V1
                     p = x < a.v1pos_n ? a.v1pos[x] : V1POS_NONE;
-                    ok = ok && p >= rlo[q] && p < rhi[q];
+                    ok = p >= rlo[q] && p < rhi[q];
                 } else {
-                    ok = dir_find(a.v1, a.g1, rlo[q], rhi[q], x, P.dir_min, p) && ok;
+                    ok = dir_find(a.v1, a.g1, rlo[q], rhi[q], x, P.dir_min, p);
                 }
                 pos[q] = p;
             }
         }
-        if (!WRITE) {
-            flags[t] = ok ? 1u : 0u;
-            continue;
-        }
-        const uint64_t e = flagoff[t];
-        e_cell[e] = c;
-        e_x[e] = x;
+    }
+    uint64_t units = 0;
+    if (ok) {
 #pragma unroll
         for (int q = 0; q < MAXOPEN; ++q) {
-            uint32_t a0 = 0, a1 = 0;
+            rlo[q] = rhi[q] = 0;
             if (q < n0) {
                 const DAtom& a = P.atom[P.src_atom[0][q]];
-                a0 = a.o1[pos[q]];
-                a1 = a.o1[pos[q] + 1];
+                rlo[q] = a.o1[pos[q]];
+                rhi[q] = a.o1[pos[q] + 1];
             }
-            rlo[q] = a0;
-            rhi[q] = a1;
-            e_rng[e * (2 * MAXOPEN) + 2 * q] = a0;
-            e_rng[e * (2 * MAXOPEN) + 2 * q + 1] = a1;
         }
-        uint32_t m = 1;  // a one-loop query: the entry is the output
+        m = 1;  // a one-loop query: the entry is the output
         if (P.nlev > 1) {
             m = 0xFFFFFFFFu;
             for (int q = 0; q < P.nsrc[1]; ++q) {
@@ -248,11 +262,8 @@ __global__ void l0_probe_kernel(const DPlan* __restrict__ gP, const uint64_t* __
                 m = min(m, len);
             }
         }
-        // work units of the entry: loop-2 candidates, each cut into slices of
-        // its loop-3 candidates when the entry fixes a long loop-3 list
-        uint32_t split = 1;
         if (P.nlev >= 4 && P.slice_grain > 0) {
-            uint32_t w = 0xFFFFFFFFu;
+            uint32_t wl = 0xFFFFFFFFu;
             for (int q = 0; q < P.nsrc[2]; ++q) {
                 const DAtom& a = P.atom[P.src_atom[2][q]];
                 uint32_t len = 0xFFFFFFFFu;
@@ -265,19 +276,107 @@ __global__ void l0_probe_kernel(const DPlan* __restrict__ gP, const uint64_t* __
                     for (int s = 0; s < MAXOPEN; ++s)
                         if (s == a.slot) len = rhi[s] - rlo[s];
                 }
-                w = min(w, len);
+                wl = min(wl, len);
             }
-            if (w != 0xFFFFFFFFu) split = max(1u, (w + P.slice_grain - 1) / P.slice_grain);
+            if (wl != 0xFFFFFFFFu) split = max(1u, (wl + P.slice_grain - 1) / P.slice_grain);
         }
-        e_units[e] = (uint64_t)m * split;
-        e_split[e] = split;
+        units = (uint64_t)m * split;
+    }
+    const uint32_t ball = __ballot_sync(0xffffffffu, ok);
+    const uint64_t uincl = warp_incl_scan64(units);
+    if (lane == 31) {
+        sh.wcnt[w] = __popc(ball);
+        sh.wunits[w] = uincl;
+    }
+    __syncthreads();
+    if (w < 2) {  // warp 0: entries, warp 1: units
+        const uint64_t tot = warp_sum64(lane < L0_WARPS ? (w == 0 ? (uint64_t)sh.wcnt[lane] : sh.wunits[lane]) : 0);
+        uint64_t* st = J.status + (uint64_t)w * J.tiles;
+        if (lane == 0) st_relaxed(st + tile, (tile == 0 ? LB_INC : LB_AGG) | tot);
+        uint64_t excl = 0;
+        if (tile != 0) {
+            excl = warp_lookback(st, tile, &J.ctl->err, wait_ns);
+            if (lane == 0) st_relaxed(st + tile, LB_INC | (excl + tot));
+        }
+        if (lane == 0) sh.excl[w] = excl;
+    }
+    __syncthreads();
+    uint64_t e = sh.excl[0], u = sh.excl[1];
+    for (uint32_t q = 0; q < w; ++q) {
+        e += sh.wcnt[q];
+        u += sh.wunits[q];
+    }
+    e += __popc(ball & lanemask_lt());
+    u += uincl - units;
+    if (ok) {
+        J.e_cell[e] = c;
+        J.e_x[e] = x;
+        J.e_split[e] = split;
+        J.uoff[e] = u;
+        uint4* rng = reinterpret_cast<uint4*>(J.e_rng + e * (2 * MAXOPEN));
+        rng[0] = make_uint4(rlo[0], rhi[0], rlo[1], rhi[1]);
+        rng[1] = make_uint4(rlo[2], rhi[2], rlo[3], rhi[3]);
+    }
+    if (tid == L0_TILE - 1 && base + L0_TILE >= T) {  // the tile of the last candidate
+        e += ok ? 1 : 0;
+        u += units;
+        J.uoff[e] = u;
+        J.ctl->n_entries = (uint32_t)e;
+    }
+    return true;
+}
+
+// Loop 1 of one query: persistent blocks take tiles in order.  The plan comes
+// as a parameter, and block 0 leaves the device copy that the search kernel
+// reads, so no copy is enqueued for it.
+__global__ void __launch_bounds__(L0_TILE) l0_kernel(const __grid_constant__ DPlan plan, L0Job J, DPlan* d_plan,
+                                                      uint32_t* tile_counter, uint64_t wait_ns) {
+    __shared__ DPlan P;
+    __shared__ L0Shared sh;
+    __shared__ uint32_t s_tile;
+    for (uint32_t i = threadIdx.x; i < sizeof(DPlan) / 4; i += blockDim.x) {
+        const uint32_t v = ((const uint32_t*)&plan)[i];
+        ((uint32_t*)&P)[i] = v;
+        if (blockIdx.x == 0) ((uint32_t*)d_plan)[i] = v;
+    }
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_tile = atomicAdd(tile_counter, 1u);
+        __syncthreads();
+        const uint32_t tile = s_tile;
+        if (tile >= J.tiles || !l0_tile(P, J, tile, wait_ns, sh)) break;
     }
 }
 
-__global__ void entries_total_kernel(const uint64_t* __restrict__ flagoff, const uint64_t* __restrict__ candoff,
-                                     uint32_t ncells, uint64_t tmax, JoinCtl* ctl) {
-    const uint64_t T = min(tmax, candoff[ncells]);
-    ctl->n_entries = (uint32_t)flagoff[T];
+// Loop 1 of all queries of a batch in one launch: the queries' tiles form one
+// sequence, handed out in order (96 small queries took 7 launches each).
+__global__ void __launch_bounds__(L0_TILE) l0_batch_kernel(const L0Job* __restrict__ jobs, uint32_t njobs,
+                                                            uint32_t tiles, uint32_t* tile_counter, uint64_t wait_ns) {
+    __shared__ DPlan P;
+    __shared__ L0Shared sh;
+    __shared__ uint32_t s_tile;
+    uint32_t cur = 0xFFFFFFFFu;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_tile = atomicAdd(tile_counter, 1u);
+        __syncthreads();
+        const uint32_t tile = s_tile;
+        if (tile >= tiles) break;
+        uint32_t lo = 0, hi = njobs;  // last job with tile0 <= tile
+        while (hi - lo > 1) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (jobs[mid].tile0 <= tile)
+                lo = mid;
+            else
+                hi = mid;
+        }
+        if (lo != cur) {
+            load_plan(P, jobs[lo].plan);
+            cur = lo;
+        }
+        const L0Job J = jobs[lo];
+        l0_tile(P, J, tile - J.tile0, wait_ns, sh);
+    }
 }
 
 // ---------------------------------------------------------- search loops
@@ -1934,61 +2033,83 @@ hc_status plan_query(const hc_query* q, const hc_index* const* idx, const hc_joi
     return HC_OK;
 }
 
-// Device buffers of one query's loop-1 pass.  The first group is needed by
-// the search; the second only during the loop-1 pass.
+// Device buffers of one query's loop-1 pass and entries, carved from one
+// allocation; the per-cell arrays, in another, exist only with several cells
+// or stats.
 struct Level1 {
     DPlan* d_plan = nullptr;
     uint32_t *e_cell = nullptr, *e_x = nullptr, *e_rng = nullptr, *e_split = nullptr;
     uint64_t* uoff = nullptr;
-    uint32_t *cand = nullptr, *flags = nullptr;
-    uint64_t *candoff = nullptr, *flagoff = nullptr, *e_units = nullptr;
+    uint32_t* cand = nullptr;
+    uint64_t* candoff = nullptr;
 };
+
+static bool needs_cells(const QueryPlan& qp) { return qp.ncells > 1 || qp.stats; }
+static uint32_t l0_tiles(const QueryPlan& qp) { return (uint32_t)((qp.cand_bound + L0_TILE - 1) / L0_TILE); }
 
 template <class Alloc>
 hc_status alloc_level1_keep(const QueryPlan& qp, Alloc& a, Level1* L) {
     const uint64_t cb = qp.cand_bound;
-    HC_TRY(a.get(&L->d_plan, 1));
-    HC_TRY(a.get(&L->e_cell, cb));
-    HC_TRY(a.get(&L->e_x, cb));
-    HC_TRY(a.get(&L->e_rng, cb * 2 * MAXOPEN));
-    HC_TRY(a.get(&L->e_split, cb));
-    HC_TRY(a.get(&L->uoff, cb + 1));
+    const uint64_t up = (cb + 3) / 4 * 4;  // arrays of up words start on 16 bytes
+    const uint64_t plan_words = (sizeof(DPlan) + 15) / 16 * 4;
+    uint32_t* p;
+    HC_TRY(a.get(&p, plan_words + up * (3 + 2 * MAXOPEN) + 2 * (cb + 1)));
+    L->d_plan = (DPlan*)p;
+    p += plan_words;
+    L->e_rng = p;
+    p += up * 2 * MAXOPEN;
+    L->e_cell = p;
+    L->e_x = p + up;
+    L->e_split = p + 2 * up;
+    L->uoff = (uint64_t*)(p + 3 * up);
     return HC_OK;
 }
 
 template <class Alloc>
-hc_status alloc_level1_temp(const QueryPlan& qp, Alloc& a, Level1* L) {
-    const uint64_t cb = qp.cand_bound;
-    HC_TRY(a.get(&L->cand, qp.ncells));
-    HC_TRY(a.get(&L->candoff, qp.ncells + 1));
-    HC_TRY(a.get(&L->flags, cb));
-    HC_TRY(a.get(&L->flagoff, cb + 1));
-    HC_TRY(a.get(&L->e_units, cb));
+hc_status alloc_level1_cells(uint64_t ncells, Alloc& a, Level1* L) {
+    HC_TRY(a.get(&L->cand, ncells));
+    HC_TRY(a.get(&L->candoff, ncells + 1));
     return HC_OK;
 }
 
-// Loop 1 of every cell (enqueued, no host waits): candidates per cell, the
-// flat probe, compaction into entries and the entries' unit offsets.  The
-// plan must already be in L.d_plan.
-hc_status enqueue_level1(const QueryPlan& qp, const Level1& L, JoinCtl* ctl, cudaStream_t s,
-                         uint64_t* cell_prof = nullptr) {
+// The query's loop-1 job.  With one cell the candidates are known here: the
+// shortest of the whole top-level lists.
+static L0Job l0_job(const QueryPlan& qp, const Level1& L, JoinCtl* ctl, uint64_t* status) {
+    L0Job J{L.d_plan, nullptr, qp.cand_bound, L.e_cell, L.e_x, L.e_rng, L.e_split, L.uoff, ctl, status, l0_tiles(qp), 0};
+    if (qp.ncells > 1) {
+        J.candoff = L.candoff;
+    } else {
+        for (int q = 0; q < qp.P.nsrc[0]; ++q)
+            J.ncand = std::min<uint64_t>(J.ncand, qp.P.atom[qp.P.src_atom[0][q]].l1_whole);
+    }
+    return J;
+}
+
+// Candidates per cell and their prefix (enqueued; the plan is in L.d_plan).
+hc_status enqueue_cells(const QueryPlan& qp, const Level1& L, JoinCtl* ctl, cudaStream_t s, uint64_t* cell_prof) {
     const int tpb = 256;
-    const uint64_t ncells = qp.ncells, cb = qp.cand_bound;
+    const uint64_t ncells = qp.ncells;
     l0_count_kernel<<<(unsigned)std::min<uint64_t>((ncells + tpb - 1) / tpb, 4096), tpb, 0, s>>>(L.d_plan, L.cand, ctl,
                                                                                                  qp.stats, cell_prof);
     if (cudaError_t le = launch_check()) return cuda_fail(le, "l0_count_kernel");
-    HC_TRY(exclusive_scan_u32_to_u64(L.cand, L.candoff, ncells, nullptr, &ctl->err, s));
-    const unsigned pgrid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((cb + tpb - 1) / tpb, (uint64_t)num_sms() * 16));
-    l0_probe_kernel<false><<<pgrid, tpb, 0, s>>>(L.d_plan, L.candoff, cb, L.flags, nullptr, nullptr, nullptr, nullptr,
-                                                 nullptr, nullptr, ctl);
-    if (cudaError_t le = launch_check()) return cuda_fail(le, "l0_probe_kernel");
-    HC_TRY(exclusive_scan_u32_to_u64(L.flags, L.flagoff, cb, nullptr, &ctl->err, s));
-    l0_probe_kernel<true><<<pgrid, tpb, 0, s>>>(L.d_plan, L.candoff, cb, L.flags, L.flagoff, L.e_cell, L.e_x, L.e_rng,
-                                                L.e_units, L.e_split, ctl);
-    if (cudaError_t le = launch_check()) return cuda_fail(le, "l0_probe_kernel");
-    entries_total_kernel<<<1, 1, 0, s>>>(L.flagoff, L.candoff, (uint32_t)ncells, cb, ctl);
-    if (cudaError_t le = launch_check()) return cuda_fail(le, "entries_total_kernel");
-    HC_TRY(exclusive_scan_u64(L.e_units, L.uoff, cb, &ctl->n_entries, &ctl->err, s));
+    return exclusive_scan_u32_to_u64(L.cand, L.candoff, ncells, nullptr, &ctl->err, s);
+}
+
+// Loop 1 of every cell (enqueued, no host waits): candidates per cell where
+// there are several, then probing, compaction into entries and their unit
+// offsets in one pass.  status (zeroed): a tile counter, then the look-back
+// words.
+hc_status enqueue_level1(const QueryPlan& qp, const Level1& L, JoinCtl* ctl, uint64_t* status, cudaStream_t s,
+                         uint64_t* cell_prof) {
+    if (needs_cells(qp)) {
+        if (cudaMemcpyAsync(L.d_plan, &qp.P, sizeof(DPlan), cudaMemcpyHostToDevice, s) != cudaSuccess)
+            return cuda_fail(cudaGetLastError(), "plan copy");
+        HC_TRY(enqueue_cells(qp, L, ctl, s, cell_prof));
+    }
+    const L0Job J = l0_job(qp, L, ctl, status + 1);
+    const unsigned grid = std::min<unsigned>(J.tiles, (unsigned)num_sms() * 6);
+    l0_kernel<<<grid, L0_TILE, 0, s>>>(qp.P, J, L.d_plan, (uint32_t*)status, wait_limit_ns());
+    if (cudaError_t le = launch_check()) return cuda_fail(le, "l0_kernel");
     return HC_OK;
 }
 
@@ -2020,10 +2141,9 @@ hc_status join_footprint_impl(const hc_query* q, const hc_index* const* idx, con
         }
         cb = std::max<uint64_t>(c, 1);
     }
-    // loop-1 buffers (kept and temporary), per-cell arrays, scan look-back
-    // words and the control block
-    const uint64_t per_cand = 4 + 4 + 4 * 2 * MAXOPEN + 4 + 8 + 4 + 8 + 8;
-    *bytes = part_bytes + cb * per_cand + qp.ncells * (4 + 8 + 8) + ((cb + 2047) / 2048) * 8 * 3 + 65536 +
+    // entries, look-back words, per-cell arrays and the control block
+    const uint64_t per_cand = 4 + 4 + 4 * 2 * MAXOPEN + 4 + 8;
+    *bytes = part_bytes + cb * per_cand + (cb / L0_TILE + 1) * 16 + qp.ncells * (4 + 8 + 8) + 65536 +
              4 * lift_arena_words(qp);
     return HC_OK;
 }
@@ -2090,13 +2210,17 @@ hc_status run_join_impl(const hc_query* q, const hc_index* const* idx, const hc_
         result_release(R);
         return st;
     };
+    // the control block, and behind it the loop-1 pass's tile counter and
+    // look-back words, cleared together
+    static_assert(sizeof(JoinCtl) % 8 == 0, "the words behind the control block are 8-byte aligned");
     {
         void* p;
-        if (dev_alloc(&p, sizeof(JoinCtl), s) != HC_OK) return bail(HC_ERR_OOM);
+        const size_t bytes = sizeof(JoinCtl) + (1 + 2 * (size_t)l0_tiles(qp)) * 8;
+        if (dev_alloc(&p, bytes, s) != HC_OK) return bail(HC_ERR_OOM);
         R->d_ctl = (JoinCtl*)p;
+        if (cudaMemsetAsync(p, 0, bytes, s) != cudaSuccess) return bail(cuda_fail(cudaGetLastError(), "memset"));
     }
     JoinCtl* ctl = R->d_ctl;
-    if (cudaMemsetAsync(ctl, 0, sizeof(JoinCtl), s) != cudaSuccess) return bail(cuda_fail(cudaGetLastError(), "memset"));
     if (prm->flags & HC_FLAG_CELL_COUNTS) {
         void* p;
         if (dev_alloc(&p, ncells * 8, s) != HC_OK) return bail(HC_ERR_OOM);
@@ -2114,10 +2238,8 @@ hc_status run_join_impl(const hc_query* q, const hc_index* const* idx, const hc_
     Level1 L;
     hc_status st;
     if ((st = alloc_level1_keep(qp, tmp, &L)) != HC_OK) return bail(st);
-    if ((st = alloc_level1_temp(qp, tmp, &L)) != HC_OK) return bail(st);
-    if (cudaMemcpyAsync(L.d_plan, &qp.P, sizeof(DPlan), cudaMemcpyHostToDevice, s) != cudaSuccess)
-        return bail(cuda_fail(cudaGetLastError(), "plan copy"));
-    if ((st = enqueue_level1(qp, L, ctl, s, R->d_cell_prof)) != HC_OK) return bail(st);
+    if (needs_cells(qp) && (st = alloc_level1_cells(ncells, tmp, &L)) != HC_OK) return bail(st);
+    if ((st = enqueue_level1(qp, L, ctl, (uint64_t*)(ctl + 1), s, R->d_cell_prof)) != HC_OK) return bail(st);
     const uint64_t* uoff = L.uoff;
 
     GjArgs g{L.d_plan, L.e_cell, L.e_x,   L.e_rng, L.e_split, uoff,    grain,   ctl, 0, R->d_cell_counts,
@@ -2365,7 +2487,10 @@ struct hc_batch {
     uint64_t* d_items = nullptr;
     uint64_t* d_item_off = nullptr;
     uint32_t* d_ctr = nullptr;
-    hc::Level1 temp;  // loop-1 temporaries shared by the queries (sized by the largest)
+    hc::Level1 temp;  // per-cell arrays shared by the queries of several cells (sized by the largest)
+    hc::L0Job* d_jobs = nullptr;
+    uint64_t* d_status = nullptr;  // look-back words of all queries' loop-1 tiles, [2 * l0_tiles]
+    uint32_t l0_tiles = 0;         // loop-1 tiles of all queries
     int class_a = 0, class_b = 0;
     bool all_shapes = false;  // more than two shape classes: gj_batch_all_kernel
     uint32_t* d_arena = nullptr;  // lifted lists (query rewriting), arena_stride words per warp
@@ -2403,7 +2528,7 @@ hc_status batch_create(const hc_query* qs, const hc_index* const* idx_flat, cons
     OwnedAlloc A{&B->mem};
     size_t off = 0;
     int classes[2] = {-1, -1};
-    uint64_t max_cb = 1, max_cells = 1;
+    uint64_t max_cells = 0, tiles = 0;
     std::vector<BQuery> hq(n);
     for (uint32_t i = 0; i < n; ++i) {
         if (prm[i].mode != HC_MODE_COUNT) return bail(fail(HC_ERR_ARG, "batch: queries run in count mode"));
@@ -2423,29 +2548,44 @@ hc_status batch_create(const hc_query* qs, const hc_index* const* idx_flat, cons
         else
             B->all_shapes = true;  // three or four shape classes: the all-shapes kernel
         if ((st = alloc_level1_keep(B->plans[i], A, &B->l1[i])) != HC_OK) return bail(st);
-        max_cb = std::max(max_cb, B->plans[i].cand_bound);
-        max_cells = std::max(max_cells, B->plans[i].ncells);
+        tiles += l0_tiles(B->plans[i]);
+        if (needs_cells(B->plans[i])) max_cells = std::max(max_cells, B->plans[i].ncells);
         if (cudaMemcpy(B->l1[i].d_plan, &B->plans[i].P, sizeof(DPlan), cudaMemcpyHostToDevice) != cudaSuccess)
             return bail(cuda_fail(cudaGetLastError(), "batch plan copy"));
     }
     if (classes[1] < 0) classes[1] = classes[0];
     B->class_a = std::min(classes[0], classes[1]);
     B->class_b = std::max(classes[0], classes[1]);
-    {
-        QueryPlan big;
-        big.cand_bound = max_cb;
-        big.ncells = max_cells;
-        hc_status st = alloc_level1_temp(big, A, &B->temp);
-        if (st != HC_OK) return bail(st);
-    }
+    if (tiles >= 0xFFFFFFFFull) return bail(fail(HC_ERR_CAPACITY, "batch: too many loop-1 candidates"));
+    B->l0_tiles = (uint32_t)tiles;
     hc_status st;
+    // cells' candidate offsets are read by the one loop-1 launch: each query
+    // of several cells keeps its own, the counts are shared
+    if (max_cells > 0) {
+        if ((st = A.get(&B->temp.cand, max_cells)) != HC_OK) return bail(st);
+        for (uint32_t i = 0; i < n; ++i)
+            if (needs_cells(B->plans[i]) && (st = A.get(&B->l1[i].candoff, B->plans[i].ncells + 1)) != HC_OK)
+                return bail(st);
+    }
     if (B->arena_stride) {  // one arena per warp of the largest batched grid (16 blocks of 4 warps per SM)
         if ((st = A.get(&B->d_arena, (size_t)num_sms() * 16 * 4 * B->arena_stride)) != HC_OK) return bail(st);
     }
     if ((st = A.get(&B->d_ctl, n)) != HC_OK || (st = A.get(&B->d_q, n)) != HC_OK ||
         (st = A.get(&B->d_items, n)) != HC_OK || (st = A.get(&B->d_item_off, (size_t)n + 1)) != HC_OK ||
-        (st = A.get(&B->d_ctr, 1)) != HC_OK)
+        (st = A.get(&B->d_ctr, 2)) != HC_OK || (st = A.get(&B->d_jobs, n)) != HC_OK ||
+        (st = A.get(&B->d_status, 2 * (size_t)tiles)) != HC_OK)
         return bail(st);
+    std::vector<L0Job> jobs(n);
+    uint64_t* status = B->d_status;
+    uint32_t tile0 = 0;
+    for (uint32_t i = 0; i < n; ++i) {
+        jobs[i] = l0_job(B->plans[i], B->l1[i], B->d_ctl + i, status);
+        jobs[i].tile0 = tile0;
+        tile0 += jobs[i].tiles;
+        status += 2 * (size_t)jobs[i].tiles;
+    }
+    if (cudaMemcpy(B->d_jobs, jobs.data(), n * sizeof(L0Job), cudaMemcpyHostToDevice) != cudaSuccess)
+        return bail(cuda_fail(cudaGetLastError(), "batch job copy"));
     for (uint32_t i = 0; i < n; ++i) {
         const Level1& L = B->l1[i];
         const int cls = shape_class(B->plans[i]);
@@ -2461,16 +2601,17 @@ hc_status batch_create(const hc_query* qs, const hc_index* const* idx_flat, cons
 
 static hc_status batch_enqueue(hc_batch* B, cudaStream_t s) {
     HC_CUDA_TRY(cudaMemsetAsync(B->d_ctl, 0, B->n * sizeof(JoinCtl), s));
-    HC_CUDA_TRY(cudaMemsetAsync(B->d_ctr, 0, sizeof(uint32_t), s));
+    HC_CUDA_TRY(cudaMemsetAsync(B->d_ctr, 0, 2 * sizeof(uint32_t), s));
+    HC_CUDA_TRY(cudaMemsetAsync(B->d_status, 0, 2 * (size_t)B->l0_tiles * sizeof(uint64_t), s));
     for (uint32_t i = 0; i < B->n; ++i) {
+        if (!needs_cells(B->plans[i])) continue;
         Level1 L = B->l1[i];
         L.cand = B->temp.cand;
-        L.candoff = B->temp.candoff;
-        L.flags = B->temp.flags;
-        L.flagoff = B->temp.flagoff;
-        L.e_units = B->temp.e_units;
-        HC_TRY(enqueue_level1(B->plans[i], L, B->d_ctl + i, s));
+        HC_TRY(enqueue_cells(B->plans[i], L, B->d_ctl + i, s, nullptr));
     }
+    l0_batch_kernel<<<std::min<unsigned>(B->l0_tiles, (unsigned)num_sms() * 6), L0_TILE, 0, s>>>(
+        B->d_jobs, B->n, B->l0_tiles, B->d_ctr + 1, wait_limit_ns());
+    HC_CUDA_TRY(launch_check());
     batch_items_kernel<<<(B->n + 255) / 256, 256, 0, s>>>(B->d_q, B->n, B->d_items);
     HC_CUDA_TRY(launch_check());
     HC_TRY(exclusive_scan_u64(B->d_items, B->d_item_off, B->n, nullptr, &B->d_ctl[0].err, s));

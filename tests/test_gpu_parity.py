@@ -474,3 +474,32 @@ def test_directory_thresholds(hc, qname, scramble):
                 r = _run(hc, q, rels, dir_min=dmin, pair_min=pmin, mode="materialize", shares=[2] * q.n_vars,
                          out_capacity=cap, merge_min=0xFFFFFFFF)
                 assert np.array_equal(sorted_rows(u32(r.tuples)), sorted_rows(ref)), (dmin, pmin, cap)
+
+
+@pytest.mark.parametrize("n", [1, 255, 256, 257, 513, 8193])
+def test_loop1_tile_edges(hc, n):
+    """Loop 1 writes its entries in tiles of 256 candidates: first lists around
+    a tile's edge (and past one block's 32 tiles), all or a third of them
+    matching, in one cell and in several, alone and in one batch."""
+    rng = np.random.default_rng(n)
+    x = np.arange(n, dtype=np.uint32) * np.uint32(3)
+    fan = [np.stack([x, (x * np.uint32(7) + np.uint32(k * 11)) % np.uint32(50)], axis=1) for k in range(3)]
+    r = np.unique(np.concatenate(fan).astype(np.uint32), axis=0)
+    s = np.unique(rng.integers(0, 50, size=(700, 2)).astype(np.uint32), axis=0)
+    t = r[r[:, 0] % 9 == 0] if n > 2 else r
+    qs, ixs, want = [], [], []
+    for rels in ([r, s, r], [r, s, t]):
+        cnt = oracle.gj_count(3, list(hc.TRIANGLE.atoms), rels)[0]
+        for sh in ([1, 1, 1], [4, 1, 1], [2, 3, 1]):
+            assert _run(hc, hc.TRIANGLE, rels, shares=sh).count == cnt, (n, sh)
+        res = _run(hc, hc.TRIANGLE, rels, mode="materialize")
+        assert res.count == cnt and res.tuples.shape[0] == cnt
+        qs.append(hc.TRIANGLE)
+        ixs.append([hc.build_index(dev(y), 0) for y in rels])
+        want.append(cnt)
+    opts = [{}, {"shares": [5, 1, 1]}]
+    b = hc.Batch(qs, ixs, opts)
+    b.launch()
+    assert b.counts() == want
+    b.launch()
+    assert b.counts() == want
