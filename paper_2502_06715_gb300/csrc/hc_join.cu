@@ -2394,6 +2394,11 @@ hc_status run_join_impl(const hc_query* q, const hc_index* const* idx, const hc_
         return HC_OK;
     }
     g.pass = 1;
+    // all items, through the pass's own counter (a single pass that overflowed
+    // leaves its segment's, which is used up)
+    g.item_lo = 0;
+    g.item_hi = 0xFFFFFFFFu;
+    g.item_ctr = nullptr;
     g.chunk_fill = nullptr;
     g.n_chunks = 0;
     g.item_counts = nullptr;

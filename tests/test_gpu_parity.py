@@ -503,3 +503,20 @@ def test_loop1_tile_edges(hc, n):
     assert b.counts() == want
     b.launch()
     assert b.counts() == want
+
+
+def test_single_pass_overflow_reruns_every_item(hc):
+    """An output larger than the pool (36 M tuples against room for one and a
+    chunk per warp): the second pass writes every item's tuples."""
+    import torch
+
+    m = 6000
+    r = np.stack([np.arange(m), np.full(m, 7)], axis=1).astype(np.uint32)
+    s = np.stack([np.full(m, 7), np.arange(m) + 10], axis=1).astype(np.uint32)
+    q = hc.Query(3, ((0, 1), (1, 2)))
+    res = hc.run_join(q, [hc.build_index(dev(r), 0), hc.build_index(dev(s), 0)], mode="materialize", out_capacity=1)
+    assert res.count == m * m and tuple(res.tuples.shape) == (m * m, 3)
+    t = res.tuples.to(torch.int64)
+    assert bool((t[:, 1] == 7).all())
+    keys = torch.sort(t[:, 0] * m + (t[:, 2] - 10)).values
+    assert bool((keys == torch.arange(m * m, device=keys.device)).all())
