@@ -285,7 +285,8 @@ typedef struct {
     uint32_t seeds[HC_MAX_VARS];  /* hash seed per variable id                          */
     uint32_t mode;                /* HC_MODE_COUNT or HC_MODE_MATERIALIZE               */
     uint32_t flags;               /* HC_FLAG_*                                          */
-    uint32_t item_grain;          /* loop-2 candidates per work item (0: default)       */
+    uint32_t item_grain;          /* loop-2 candidates (or slices) per work item (0: up  */
+                                  /* to 64, fewer when the launch's warps need the items) */
     uint32_t block_threads;       /* threads per block of the search kernel, a multiple */
                                   /* of 32 up to 128 (0: default 128)                   */
     uint32_t merge_min;           /* last loop: two lists both at least this long ...   */

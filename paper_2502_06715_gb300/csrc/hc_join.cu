@@ -397,6 +397,23 @@ struct Entry {
     uint32_t j0, j1, ns;   // slices [j0, j1) of ns of the loop-2 binding's loop-3 candidates
 };
 
+// Work units per item when the caller names none: enough items for every warp
+// of the launch to take several, so that the warps end together, between a
+// lower bound and 64.  A unit of a 3-loop query is one list intersection per
+// candidate, and four candidates keep a round's lanes and its memory reads
+// busy; a unit of a deeper query carries a whole subtree of a hub or almost
+// nothing, so its items may be single units and more of them are wanted.
+// With 64 always, small and skewed graphs left most of the chip idle:
+// 4-cycle on R-MAT 10 / 13 14.5 / 39.7 -> 0.74 / 19.0 ms, 4-clique on R-MAT 12
+// 3.9 -> 0.75, triangle on 4,096 vertices and 32,768 edges 0.180 -> 0.101 a
+// call; the 4-clique on R-MAT 17 (40.3 -> 38.9) and the triangle on R-MAT 20
+// (7.81) are the upper end.
+__host__ __device__ inline uint32_t auto_grain(uint64_t units, uint64_t warps, int nlev) {
+    const uint64_t per = nlev >= 4 ? 16 : 4, least = nlev >= 4 ? 1 : 4;
+    const uint64_t g = units / (warps * per);
+    return (uint32_t)(g < least ? least : g > 64 ? 64 : g);
+}
+
 // Batch bindings of loops 1..NL-2 (index = loop), one per lane.
 template <int NL, int O>
 struct Frame {
@@ -1289,7 +1306,7 @@ __global__ void __launch_bounds__(128, (NL <= 3 ? 16 : 12)) gj_kernel(const DPla
                                                     const uint32_t* __restrict__ e_x,
                                                     const uint32_t* __restrict__ e_rng,
                                                     const uint32_t* __restrict__ e_split,
-                                                    const uint64_t* __restrict__ uoff, uint32_t grain, JoinCtl* ctl,
+                                                    const uint64_t* __restrict__ uoff, uint32_t grain_in, JoinCtl* ctl,
                                                     int pass, uint64_t* __restrict__ cell_counts,
                                                     uint64_t* __restrict__ item_counts,
                                                     const uint64_t* __restrict__ item_base, uint32_t* __restrict__ out,
@@ -1304,6 +1321,7 @@ __global__ void __launch_bounds__(128, (NL <= 3 ? 16 : 12)) gj_kernel(const DPla
     const uint32_t lane = lane_id();
     const uint32_t E_n = ctl->n_entries;
     const uint64_t U = uoff[E_n];
+    const uint32_t grain = grain_in ? grain_in : auto_grain(U, (uint64_t)gridDim.x * (blockDim.x >> 5), NL);
     const uint64_t nitems = (U + grain - 1) / grain;
     Frame<NL, O> F;
     F.lifted = false;
@@ -1355,15 +1373,31 @@ struct BQuery {
     const uint32_t *e_cell, *e_x, *e_rng, *e_split;
     const uint64_t* uoff;
     JoinCtl* ctl;
-    uint32_t grain;
+    uint32_t grain;  // as asked for (0: auto_grain over the batch's units)
+    uint32_t run;    // the grain of this launch (batch_items_kernel)
+    uint32_t nlev;
     uint32_t shape;  // 0: the kernel's first shape, 1: its second (all-shapes kernel: the shape class)
 };
 
-__global__ void batch_items_kernel(const BQuery* __restrict__ qs, uint32_t n, uint64_t* __restrict__ items) {
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const BQuery& b = qs[i];
+// One block: the batch's work units, from them each query's grain, and its
+// number of items.  A batch's queries end together, so twice as many items a
+// warp as a single query's are cut (96 graphs of about 30,000 edges: 13.9 ms
+// at 8 to 16 units an item, 14.5 at 32 and 16.0 at 64).
+__global__ void __launch_bounds__(1024) batch_items_kernel(BQuery* __restrict__ qs, uint32_t n, uint64_t warps,
+                                                           uint64_t* __restrict__ items) {
+    __shared__ uint64_t s_sum[32];
+    uint64_t sum = 0;
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) sum += qs[i].uoff[qs[i].ctl->n_entries];
+    sum = warp_sum64(sum);
+    if (lane_id() == 0) s_sum[threadIdx.x >> 5] = sum;
+    __syncthreads();
+    uint64_t total = 0;
+    for (uint32_t w = 0; w < 32; ++w) total += s_sum[w];
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+        BQuery& b = qs[i];
         const uint64_t U = b.uoff[b.ctl->n_entries];
-        items[i] = (U + b.grain - 1) / b.grain;
+        b.run = b.grain ? b.grain : auto_grain(total / 2, b.nlev >= 4 ? warps : 4 * warps, (int)b.nlev);
+        items[i] = (U + b.run - 1) / b.run;
     }
 }
 
@@ -1427,13 +1461,13 @@ __global__ void __launch_bounds__(128, ((NLA <= 3 && NLB <= 3) ? 16 : 12))
             Frame<NLA, OA> F;
             F.lifted = false;
             c = search_item<NLA, SA, OA, false>(P, F, A, (uint32_t(*)[SA])s_e[w], (uint32_t(*)[SA])(s_e[w] + NLA * SA),
-                                                local, b.grain, E_n, U, b.e_cell, b.e_x, b.e_rng, b.e_split, b.uoff,
+                                                local, b.run, E_n, U, b.e_cell, b.e_x, b.e_rng, b.e_split, b.uoff,
                                                 nullptr, 0);
         } else {
             Frame<NLB, OB> F;
             F.lifted = false;
             c = search_item<NLB, SB, OB, false>(P, F, A, (uint32_t(*)[SB])s_e[w], (uint32_t(*)[SB])(s_e[w] + NLB * SB),
-                                                local, b.grain, E_n, U, b.e_cell, b.e_x, b.e_rng, b.e_split, b.uoff,
+                                                local, b.run, E_n, U, b.e_cell, b.e_x, b.e_rng, b.e_split, b.uoff,
                                                 nullptr, 0);
         }
         if (lane == 0 && c) atomicAdd((unsigned long long*)&b.ctl->total, (unsigned long long)c);
@@ -1501,7 +1535,7 @@ __global__ void __launch_bounds__(128, 12)
                 Frame<3, 2> F;
                 F.lifted = false;
                 c = search_item<3, 2, 2, false>(P, F, A, (uint32_t(*)[2])s_e[w], (uint32_t(*)[2])(s_e[w] + 3 * 2),
-                                                local, b.grain, E_n, U, b.e_cell, b.e_x, b.e_rng, b.e_split, b.uoff,
+                                                local, b.run, E_n, U, b.e_cell, b.e_x, b.e_rng, b.e_split, b.uoff,
                                                 nullptr, 0);
                 break;
             }
@@ -1509,7 +1543,7 @@ __global__ void __launch_bounds__(128, 12)
                 Frame<3, 4> F;
                 F.lifted = false;
                 c = search_item<3, 4, 4, false>(P, F, A, (uint32_t(*)[4])s_e[w], (uint32_t(*)[4])(s_e[w] + 3 * 4),
-                                                local, b.grain, E_n, U, b.e_cell, b.e_x, b.e_rng, b.e_split, b.uoff,
+                                                local, b.run, E_n, U, b.e_cell, b.e_x, b.e_rng, b.e_split, b.uoff,
                                                 nullptr, 0);
                 break;
             }
@@ -1517,7 +1551,7 @@ __global__ void __launch_bounds__(128, 12)
                 Frame<4, 2> F;
                 F.lifted = false;
                 c = search_item<4, 2, 2, false>(P, F, A, (uint32_t(*)[2])s_e[w], (uint32_t(*)[2])(s_e[w] + 4 * 2),
-                                                local, b.grain, E_n, U, b.e_cell, b.e_x, b.e_rng, b.e_split, b.uoff,
+                                                local, b.run, E_n, U, b.e_cell, b.e_x, b.e_rng, b.e_split, b.uoff,
                                                 nullptr, 0);
                 break;
             }
@@ -1525,7 +1559,7 @@ __global__ void __launch_bounds__(128, 12)
                 Frame<4, 4> F;
                 F.lifted = false;
                 c = search_item<4, 4, 4, false>(P, F, A, (uint32_t(*)[4])s_e[w], (uint32_t(*)[4])(s_e[w] + 4 * 4),
-                                                local, b.grain, E_n, U, b.e_cell, b.e_x, b.e_rng, b.e_split, b.uoff,
+                                                local, b.run, E_n, U, b.e_cell, b.e_x, b.e_rng, b.e_split, b.uoff,
                                                 nullptr, 0);
                 break;
             }
@@ -1798,7 +1832,7 @@ hc_status result_get(hc_result* R, hc_result_view* v) {
 struct QueryPlan {
     DPlan P;
     int nv = 0, shape_s = 2, shape_o = 2, threads = 128, stats = 0;
-    uint32_t grain = 64;
+    uint32_t grain = 0;  // work units per item (0: auto_grain)
     uint64_t ncells = 1, cand_bound = 1;
     std::vector<hc_partitioned*> parts;
     std::vector<const hc_index*> part_src;  // the index each partitioned copy was made from
@@ -1853,7 +1887,7 @@ hc_status plan_query(const hc_query* q, const hc_index* const* idx, const hc_joi
             st *= prm->shares[v];
         }
     }
-    out->grain = prm->item_grain ? prm->item_grain : 64;
+    out->grain = prm->item_grain;
     out->threads = prm->block_threads ? (int)prm->block_threads : 128;
     if (out->threads % 32 != 0 || out->threads < 32 || out->threads > 128)
         return fail(HC_ERR_ARG, "run_join: block_threads must be a multiple of 32 in [32, 128]");
@@ -2197,7 +2231,6 @@ hc_status run_join_impl(const hc_query* q, const hc_index* const* idx, const hc_
     QueryPlan qp;
     HC_TRY(plan_query(q, idx, prm, s, &qp));
     const int nv = qp.nv, shape_s = qp.shape_s, shape_o = qp.shape_o, threads = qp.threads, stats = qp.stats;
-    const uint32_t grain = qp.grain;
     const uint64_t ncells = qp.ncells;
 
     hc_result* R = new hc_result();
@@ -2242,7 +2275,7 @@ hc_status run_join_impl(const hc_query* q, const hc_index* const* idx, const hc_
     if ((st = enqueue_level1(qp, L, ctl, (uint64_t*)(ctl + 1), s, R->d_cell_prof)) != HC_OK) return bail(st);
     const uint64_t* uoff = L.uoff;
 
-    GjArgs g{L.d_plan, L.e_cell, L.e_x,   L.e_rng, L.e_split, uoff,    grain,   ctl, 0, R->d_cell_counts,
+    GjArgs g{L.d_plan, L.e_cell, L.e_x,   L.e_rng, L.e_split, uoff,    qp.grain, ctl, 0, R->d_cell_counts,
              nullptr,  nullptr,  nullptr, stats,   threads,   nullptr, 0};
     if (const uint64_t aw = lift_arena_words(qp)) {
         if ((st = tmp.get(&g.arena, aw)) != HC_OK) return bail(st);
@@ -2268,6 +2301,11 @@ hc_status run_join_impl(const hc_query* q, const hc_index* const* idx, const hc_
     if (cudaMemcpyAsync(&hU, uoff + R->h_ctl.n_entries, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return bail(cuda_fail(cudaGetLastError(), "read units"));
+    // both passes cut the same items: the grain is fixed here
+    const uint32_t grain =
+        qp.grain ? qp.grain
+                 : auto_grain(hU, (uint64_t)gj_grid_any(nv, shape_s, shape_o, false, threads) * (threads / 32), nv);
+    g.grain = grain;
     const uint64_t nitems = (hU + grain - 1) / grain;
     R->n_items = nitems;
     uint64_t *item_counts, *item_base;
@@ -2595,7 +2633,7 @@ hc_status batch_create(const hc_query* qs, const hc_index* const* idx_flat, cons
         const Level1& L = B->l1[i];
         const int cls = shape_class(B->plans[i]);
         hq[i] = BQuery{L.d_plan, L.e_cell, L.e_x, L.e_rng, L.e_split, L.uoff, B->d_ctl + i, B->plans[i].grain,
-                       (uint32_t)(B->all_shapes ? cls : (cls == B->class_a ? 0 : 1))};
+                       0u, (uint32_t)B->plans[i].nv, (uint32_t)(B->all_shapes ? cls : (cls == B->class_a ? 0 : 1))};
     }
     if (cudaMemcpy(B->d_q, hq.data(), n * sizeof(BQuery), cudaMemcpyHostToDevice) != cudaSuccess)
         return bail(cuda_fail(cudaGetLastError(), "batch table copy"));
@@ -2617,7 +2655,7 @@ static hc_status batch_enqueue(hc_batch* B, cudaStream_t s) {
     l0_batch_kernel<<<std::min<unsigned>(B->l0_tiles, (unsigned)num_sms() * 6), L0_TILE, 0, s>>>(
         B->d_jobs, B->n, B->l0_tiles, B->d_ctr + 1, wait_limit_ns());
     HC_CUDA_TRY(launch_check());
-    batch_items_kernel<<<(B->n + 255) / 256, 256, 0, s>>>(B->d_q, B->n, B->d_items);
+    batch_items_kernel<<<1, 1024, 0, s>>>(B->d_q, B->n, (uint64_t)num_sms() * 48, B->d_items);
     HC_CUDA_TRY(launch_check());
     HC_TRY(exclusive_scan_u64(B->d_items, B->d_item_off, B->n, nullptr, &B->d_ctl[0].err, s));
     if (B->all_shapes) {

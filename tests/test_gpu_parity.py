@@ -520,3 +520,26 @@ def test_single_pass_overflow_reruns_every_item(hc):
     assert bool((t[:, 1] == 7).all())
     keys = torch.sort(t[:, 0] * m + (t[:, 2] - 10)).values
     assert bool((keys == torch.arange(m * m, device=keys.device)).all())
+
+
+@pytest.mark.parametrize("qname", ["TRIANGLE", "FOUR_CYCLE", "TWO_TRIANGLE"])
+def test_default_item_grain(hc, qname):
+    """The default work items (cut by the number of work units) give what one
+    unit an item and 64 give, counted, written in both forms and batched."""
+    q = getattr(hc, qname)
+    sym = datagen.rmat_graph(7, 6, 5)
+    rel = datagen.orient_lt(sym) if qname != "FOUR_CYCLE" else sym
+    rels = [rel] * len(q.atoms)
+    ref = sorted_rows(oracle.gj_enumerate(q.n_vars, list(q.atoms), rels))
+    for grain in (0, 1, 64):
+        for sh in ([1] * q.n_vars, [2] + [1] * (q.n_vars - 1)):
+            assert _run(hc, q, rels, item_grain=grain, shares=sh).count == ref.shape[0], (grain, sh)
+        for cap in (0, 2 * ref.shape[0] + 1):
+            got = u32(_run(hc, q, rels, item_grain=grain, mode="materialize", out_capacity=cap).tuples)
+            assert np.array_equal(sorted_rows(got), ref), (grain, cap)
+    if q.n_vars <= 4:
+        ix = {o: hc.build_index(dev(rel), o) for o in (0, 1)}
+        lst = [ix[q.attr_order(j)] for j in range(len(q.atoms))]
+        b = hc.Batch([q] * 3, [lst] * 3, [{}, {"item_grain": 1}, {"item_grain": 64}])
+        b.launch()
+        assert b.counts() == [ref.shape[0]] * 3
