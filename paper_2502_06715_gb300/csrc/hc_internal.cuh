@@ -432,12 +432,15 @@ __device__ __forceinline__ Dense dense_of(uint32_t lo, uint32_t hi, uint32_t vmi
 #endif  // __CUDACC__
 
 // --------------------------------------------------------------- host entry
-// Sorting and CoCo construction (hc_sort.cu).  BUILD_NO_DIRECTORIES (a
-// flag of internal callers that only want the sorted keys) skips the
-// position map and the bucket directories.
-constexpr uint32_t BUILD_NO_DIRECTORIES = 0x80000000u;
+// Sorting and CoCo construction (hc_sort.cu).
 hc_status build_index_impl(const uint32_t* d_pairs, uint64_t n, uint32_t attr_order, uint32_t flags,
                            cudaStream_t s, hc_index** out);
+// d_pairs sorted by (first, second) into keys (first << 32 | second, [n]
+// allocated here), the largest values being known; enqueued without waiting.
+// A look-back that gives up sets DEV_ERR_TIMEOUT in *d_err, after which the
+// keys are not valid.
+hc_status sort_pairs(const uint2* d_pairs, uint64_t n, uint32_t max_first, uint32_t max_second, uint32_t* d_err,
+                     cudaStream_t s, uint64_t** out_keys);
 hc_status partition_impl(const hc_index* idx, uint32_t seed_a, uint32_t pa, uint32_t seed_b,
                          uint32_t pb, cudaStream_t s, hc_partitioned** out);
 void partitioned_release(hc_partitioned* p, cudaStream_t s);

@@ -195,7 +195,9 @@ __global__ void kpack_kernel(const uint32_t* __restrict__ rows, uint64_t n, KLay
 // Pairs (value of column `col` of row perm[i], i) for one level pass of the
 // unpacked sort (perm NULL: the identity).
 __global__ void kperm_pairs_kernel(const uint32_t* __restrict__ rows, uint64_t n, uint32_t k, uint32_t col,
-                                   const uint32_t* __restrict__ perm, uint2* __restrict__ out) {
+                                   const uint32_t* __restrict__ perm, uint2* __restrict__ out,
+                                   const uint32_t* __restrict__ err) {
+    if (dev_err_set(err)) return;  // a sort pass gave up a wait: perm is not an order of the rows
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t r = perm ? perm[i] : i;
         out[i] = make_uint2(rows[r * k + col], (uint32_t)i);
@@ -205,7 +207,9 @@ __global__ void kperm_pairs_kernel(const uint32_t* __restrict__ rows, uint64_t n
 // Pairs (partition id of row perm[i], i): the last, most significant pass of
 // a partitioned unpacked sort.
 __global__ void kpid_pairs_kernel(const uint32_t* __restrict__ rows, uint64_t n, KLayout L, KPart Pt,
-                                  const uint32_t* __restrict__ perm, uint2* __restrict__ out) {
+                                  const uint32_t* __restrict__ perm, uint2* __restrict__ out,
+                                  const uint32_t* __restrict__ err) {
+    if (dev_err_set(err)) return;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t r = perm ? perm[i] : i;
         uint32_t pid = 0;
@@ -219,7 +223,8 @@ __global__ void kpid_pairs_kernel(const uint32_t* __restrict__ rows, uint64_t n,
 // After a pass sorted the pairs: the new order is the old order read at the
 // positions the sorted keys carry in their low words.
 __global__ void kperm_compose_kernel(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ perm_old,
-                                     uint32_t* __restrict__ perm_new, uint64_t n) {
+                                     uint32_t* __restrict__ perm_new, uint64_t n, const uint32_t* __restrict__ err) {
+    if (dev_err_set(err)) return;  // the keys are not sorted pairs
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t j = (uint32_t)keys[i];
         perm_new[i] = perm_old ? perm_old[j] : j;
@@ -586,9 +591,13 @@ hc_status build_kindex_impl(const uint32_t* d_rows, uint64_t n, uint32_t k, cons
     src.part = Pt;
     src.bpref = x->d_bpref;
     src.l0start = x->d_l0start;
-    hc_index* sorted = nullptr;  // holds the packed keys, sorted
+    // The passes' maxima are known and their errors go to ctl, so nothing is
+    // waited for or built beside the sorted keys (going through the binary
+    // index's builder read the keys twice more, and waited twice: 8 % of
+    // indexing the 19 M triangles of R-MAT 17).
+    uint64_t* keys = nullptr;  // sorted
     auto bail2 = [&](hc_status e) {
-        if (sorted) index_release(sorted, s);
+        dev_free(keys, s);
         destroy_events();
         return bail(e);
     };
@@ -598,37 +607,31 @@ hc_status build_kindex_impl(const uint32_t* d_rows, uint64_t n, uint32_t k, cons
         if ((st = tmp.get(&pk, n)) != HC_OK) return bail2(st);
         kpack_kernel<<<grid_of(n, 256, 8), 256, 0, s>>>(d_rows, n, L, Pt, total_bits, pk);
         if (cudaError_t le = launch_check()) return bail2(cuda_fail(le, "kpack_kernel"));
-        if ((st = build_index_impl((const uint32_t*)pk, n, 0, BUILD_NO_DIRECTORIES, s, &sorted)) != HC_OK) return bail2(st);
-        src.keys = sorted->d_keys;
+        const uint32_t kb = total_bits + pid_bits;  // the packed key's bits, above and below bit 32
+        const uint32_t hi = kb > 32 ? (uint32_t)((1ull << (kb - 32)) - 1) : 0u;
+        const uint32_t lo = kb >= 32 ? 0xFFFFFFFFu : (uint32_t)((1ull << kb) - 1);
+        if ((st = sort_pairs(pk, n, hi, lo, &ctl->err, s, &keys)) != HC_OK) return bail2(st);
+        src.keys = keys;
     } else {
         uint2* pairs;
         uint32_t *pa, *pb;
         if ((st = tmp.get(&pairs, n)) != HC_OK || (st = tmp.get(&pa, n)) != HC_OK || (st = tmp.get(&pb, n)) != HC_OK)
             return bail2(st);
         const uint32_t* cur = nullptr;
-        for (int d = (int)k - 1; d >= 0; --d) {
-            kperm_pairs_kernel<<<grid_of(n, 256, 8), 256, 0, s>>>(d_rows, n, k, cols[d], cur, pairs);
+        // last level first, and the partition id last: the most significant key
+        for (int d = (int)k - 1; d >= (np > 1 ? -1 : 0); --d) {
+            if (d >= 0)
+                kperm_pairs_kernel<<<grid_of(n, 256, 8), 256, 0, s>>>(d_rows, n, k, cols[d], cur, pairs, &ctl->err);
+            else
+                kpid_pairs_kernel<<<grid_of(n, 256, 8), 256, 0, s>>>(d_rows, n, L, Pt, cur, pairs, &ctl->err);
             if (cudaError_t le = launch_check()) return bail2(cuda_fail(le, "kperm_pairs_kernel"));
-            hc_index* pass = nullptr;
-            if ((st = build_index_impl((const uint32_t*)pairs, n, 0, BUILD_NO_DIRECTORIES, s, &pass)) != HC_OK) return bail2(st);
+            const uint32_t top = d >= 0 ? x->maxv[d] : (uint32_t)(np - 1);
+            if ((st = sort_pairs(pairs, n, top, (uint32_t)(n - 1), &ctl->err, s, &keys)) != HC_OK) return bail2(st);
             uint32_t* nxt = cur == pa ? pb : pa;
-            kperm_compose_kernel<<<grid_of(n, 256, 8), 256, 0, s>>>(pass->d_keys, cur, nxt, n);
-            cudaError_t le = launch_check();
-            index_release(pass, s);
-            if (le) return bail2(cuda_fail(le, "kperm_compose_kernel"));
-            cur = nxt;
-        }
-        if (np > 1) {  // the partition id last: the most significant key
-            kpid_pairs_kernel<<<grid_of(n, 256, 8), 256, 0, s>>>(d_rows, n, L, Pt, cur, pairs);
-            if (cudaError_t le = launch_check()) return bail2(cuda_fail(le, "kpid_pairs_kernel"));
-            hc_index* pass = nullptr;
-            if ((st = build_index_impl((const uint32_t*)pairs, n, 0, BUILD_NO_DIRECTORIES, s, &pass)) != HC_OK)
-                return bail2(st);
-            uint32_t* nxt = cur == pa ? pb : pa;
-            kperm_compose_kernel<<<grid_of(n, 256, 8), 256, 0, s>>>(pass->d_keys, cur, nxt, n);
-            cudaError_t le = launch_check();
-            index_release(pass, s);
-            if (le) return bail2(cuda_fail(le, "kperm_compose_kernel"));
+            kperm_compose_kernel<<<grid_of(n, 256, 8), 256, 0, s>>>(keys, cur, nxt, n, &ctl->err);
+            if (cudaError_t le = launch_check()) return bail2(cuda_fail(le, "kperm_compose_kernel"));
+            dev_free(keys, s);
+            keys = nullptr;
             cur = nxt;
         }
         src.rows = d_rows;
@@ -655,10 +658,8 @@ hc_status build_kindex_impl(const uint32_t* d_rows, uint64_t n, uint32_t k, cons
     if (cudaMemcpyAsync(&h, ctl, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return bail2(cuda_fail(cudaGetLastError(), "build_kindex: level scan"));
-    if (sorted) {
-        index_release(sorted, s);
-        sorted = nullptr;
-    }
+    dev_free(keys, s);
+    keys = nullptr;
     if (h.err & DEV_ERR_TIMEOUT) return bail2(fail(HC_ERR_TIMEOUT, "build_kindex: a look-back wait gave up"));
     if ((flags & HC_BUILD_CHECK_DUPLICATES) && h.dup)
         return bail2(fail(HC_ERR_DUPLICATE, "build_kindex: the relation holds a repeated row"));

@@ -747,8 +747,8 @@ struct LaunchTimer {
 
 // Radix passes over the given digit specs; the sorted keys end in `dst`.
 hc_status radix_passes(const void* src, bool src_pairs, uint32_t ao, uint64_t n, const std::vector<DigitSpec>& specs,
-                       uint64_t* dst, Tmp& tmp, Ctl* d_ctl, cudaStream_t s, LaunchTimer* timer = nullptr,
-                       bool withhold_first = false) {
+                       uint64_t* dst, Tmp& tmp, uint32_t* tile_counters, uint32_t* err, cudaStream_t s,
+                       LaunchTimer* timer = nullptr, bool withhold_first = false) {
     const int np = (int)specs.size();
     if (np == 0) return fail(HC_ERR_ARG, "internal: no radix passes");
     DigitSpec* d_specs;
@@ -788,7 +788,7 @@ hc_status radix_passes(const void* src, bool src_pairs, uint32_t ao, uint64_t n,
                                           : onesweep_kernel<SRC_KEYS, DIGIT_PARTITION>;
         if (timer) HC_TRY(timer->mark(s));
         kern<<<(unsigned)ntiles, PASS_THREADS, 0, s>>>(in, outb, n32, ao, specs[p], d_hist + p * RADIX, status,
-                                                       &d_ctl->tile_counter[p], &d_ctl->err, wait_limit_ns(),
+                                                       tile_counters + p, err, wait_limit_ns(),
                                                        (withhold_first && p == 0) ? 1u : 0u);
         HC_CUDA_TRY(launch_check());
         if (timer) HC_TRY(timer->mark(s));
@@ -819,6 +819,14 @@ hc_status run_boundary(const uint64_t* keys, uint64_t n, bool segmented, uint32_
 }
 
 uint32_t bits_of(uint32_t v) { return v == 0 ? 0 : 32 - __builtin_clz(v); }
+
+// The passes of a sort of keys first << 32 | second: the bytes in use.
+std::vector<DigitSpec> key_digits(uint32_t max_first, uint32_t max_second) {
+    std::vector<DigitSpec> specs;
+    for (uint32_t b = 0; b < bits_of(max_second); b += 8) specs.push_back({0, b, 0, 1, 0, 1});
+    for (uint32_t b = 0; b < bits_of(max_first); b += 8) specs.push_back({0, 32 + b, 0, 1, 0, 1});
+    return specs;
+}
 
 }  // namespace
 
@@ -917,13 +925,12 @@ hc_status build_index_impl(const uint32_t* d_pairs, uint64_t n, uint32_t ao, uin
         if ((st = check_ctl(d_ctl, s, &h)) != HC_OK) return bail(st);
         idx->max_first = ao ? h.maxv[1] : h.maxv[0];
         idx->max_second = ao ? h.maxv[0] : h.maxv[1];
-        std::vector<DigitSpec> specs;
-        for (uint32_t b = 0; b < bits_of(idx->max_second); b += 8) specs.push_back({0, b, 0, 1, 0, 1});
-        for (uint32_t b = 0; b < bits_of(idx->max_first); b += 8) specs.push_back({0, 32 + b, 0, 1, 0, 1});
+        const std::vector<DigitSpec> specs = key_digits(idx->max_first, idx->max_second);
         if (specs.empty()) {
             pack_kernel<<<grid_for(n, 256, 4), 256, 0, s>>>((const uint2*)d_pairs, idx->d_keys, n, ao);
             if (cudaError_t le = launch_check()) return bail(cuda_fail(le, "pack_kernel"));
-        } else if ((st = radix_passes(d_pairs, true, ao, n, specs, idx->d_keys, tmp, d_ctl, s, &t_radix,
+        } else if ((st = radix_passes(d_pairs, true, ao, n, specs, idx->d_keys, tmp, d_ctl->tile_counter, &d_ctl->err, s,
+                                      &t_radix,
                                       (flags & HC_BUILD_TEST_STALL_SORT) != 0)) != HC_OK) {
             return bail(st);
         }
@@ -944,10 +951,6 @@ hc_status build_index_impl(const uint32_t* d_pairs, uint64_t n, uint32_t ao, uin
             return bail(fail(HC_ERR_DUPLICATE, "build_index: the relation holds a repeated row"));
         idx->l1 = h.l1;
         idx->max_run = h.maxrun;
-        if (flags & BUILD_NO_DIRECTORIES) {
-            *out = idx;
-            return HC_OK;
-        }
         if (v1pos_eligible(n, idx->max_first)) {
             const uint64_t dn = (uint64_t)idx->max_first + 1;
             if (dev_alloc(&p, dn * 4, s) != HC_OK) return bail(HC_ERR_OOM);
@@ -962,6 +965,35 @@ hc_status build_index_impl(const uint32_t* d_pairs, uint64_t n, uint32_t ao, uin
         if ((st = build_level_directories(idx, s)) != HC_OK) return bail(st);
     }
     *out = idx;
+    return HC_OK;
+}
+
+hc_status sort_pairs(const uint2* d_pairs, uint64_t n, uint32_t max_first, uint32_t max_second, uint32_t* d_err,
+                     cudaStream_t s, uint64_t** out_keys) {
+    *out_keys = nullptr;
+    void* p;
+    HC_TRY(dev_alloc(&p, std::max<uint64_t>(n, 1) * 8, s));
+    uint64_t* keys = (uint64_t*)p;
+    const std::vector<DigitSpec> specs = key_digits(max_first, max_second);
+    hc_status st = HC_OK;
+    if (specs.empty()) {
+        pack_kernel<<<grid_for(n, 256, 4), 256, 0, s>>>(d_pairs, keys, n, 0);
+        if (cudaError_t le = launch_check()) st = cuda_fail(le, "pack_kernel");
+    } else {
+        Tmp tmp(s);
+        uint32_t* counters;
+        if ((st = tmp.get(&counters, MAX_PASSES)) == HC_OK) {
+            if (cudaMemsetAsync(counters, 0, MAX_PASSES * sizeof(uint32_t), s) != cudaSuccess)
+                st = cuda_fail(cudaGetLastError(), "memset");
+            else
+                st = radix_passes(d_pairs, true, 0, n, specs, keys, tmp, counters, d_err, s);
+        }
+    }
+    if (st != HC_OK) {
+        dev_free(keys, s);
+        return st;
+    }
+    *out_keys = keys;
     return HC_OK;
 }
 
@@ -1107,7 +1139,8 @@ hc_status partition_impl(const hc_index* idx, uint32_t seed_a, uint32_t pa, uint
         } else {
             std::vector<DigitSpec> specs;
             for (uint32_t b = 0; b < bits_of(np - 1); b += 8) specs.push_back({1, b, seed_a, pa, seed_b, pb});
-            if ((st = radix_passes(idx->d_keys, false, 0, n, specs, part->d_keys, tmp, d_ctl, s)) != HC_OK)
+            if ((st = radix_passes(idx->d_keys, false, 0, n, specs, part->d_keys, tmp, d_ctl->tile_counter,
+                                   &d_ctl->err, s)) != HC_OK)
                 return bail(st);
         }
         if ((st = run_boundary(part->d_keys, n, true, seed_a, pa, seed_b, pb, part->d_v1, part->d_o1, part->d_v2, tmp,
