@@ -1387,7 +1387,9 @@ __global__ void __launch_bounds__(1024) batch_items_kernel(BQuery* __restrict__ 
                                                            uint64_t* __restrict__ items) {
     __shared__ uint64_t s_sum[32];
     uint64_t sum = 0;
-    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) sum += qs[i].uoff[qs[i].ctl->n_entries];
+    // a query whose loop-1 pass gave up a wait has no valid offsets: no items
+    const auto units = [](const BQuery& b) { return dev_err_set(&b.ctl->err) ? 0ull : b.uoff[b.ctl->n_entries]; };
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) sum += units(qs[i]);
     sum = warp_sum64(sum);
     if (lane_id() == 0) s_sum[threadIdx.x >> 5] = sum;
     __syncthreads();
@@ -1395,7 +1397,7 @@ __global__ void __launch_bounds__(1024) batch_items_kernel(BQuery* __restrict__ 
     for (uint32_t w = 0; w < 32; ++w) total += s_sum[w];
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
         BQuery& b = qs[i];
-        const uint64_t U = b.uoff[b.ctl->n_entries];
+        const uint64_t U = units(b);
         b.run = b.grain ? b.grain : auto_grain(total / 2, b.nlev >= 4 ? warps : 4 * warps, (int)b.nlev);
         items[i] = (U + b.run - 1) / b.run;
     }
