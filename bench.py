@@ -412,7 +412,7 @@ def main():
                        "shares_from": a.shares if a.shares not in ("plan", "autotune") else
                        (f"choose_shares(P={a.P})" if a.shares == "plan" else
                         f"autotune (>= {a.min_cells} cells; candidates include choose_shares(P=64..1024))"),
-                       "plan_shares_P1024": plan_shares, "item_grain": a.grain or 64,
+                       "plan_shares_P1024": plan_shares, "item_grain": a.grain or "by size",
                        "merge": [knobs.get("merge_min", 32), knobs.get("merge_ratio", 4)],
                        "dir_min": knobs["dir_min"] or 16, "pair_min": knobs["pair_min"] or 32,
                        "out_capacity": capacity if a.mode == "materialize" else None,
