@@ -413,7 +413,8 @@ def main():
                        (f"choose_shares(P={a.P})" if a.shares == "plan" else
                         f"autotune (>= {a.min_cells} cells; candidates include choose_shares(P=64..1024))"),
                        "plan_shares_P1024": plan_shares, "item_grain": a.grain or "by size",
-                       "merge": [knobs.get("merge_min", 32), knobs.get("merge_ratio", 4)],
+                       "merge": ("auto" if not (knobs.get("merge_min") or knobs.get("merge_ratio"))
+                                 else [knobs["merge_min"], knobs["merge_ratio"]]),
                        "dir_min": knobs["dir_min"] or 16, "pair_min": knobs["pair_min"] or 32,
                        "out_capacity": capacity if a.mode == "materialize" else None,
                        "search_launches_per_step": n_launch_per_step,

@@ -8,15 +8,19 @@ hand and keeps the fastest configuration, searching one knob at a time
 
   shares        the plan of ``choose_shares`` at several cell counts P, plus
                 all-on-the-first-variable and square splits of the same P;
-  item_grain    loop-2 candidates per work item;
+  item_grain    loop-2 candidates per work item, or by the join's size (0);
   merge         when the last loop uses the warp merge path (min length,
-                length ratio) or never;
+                length ratio), never, or by what the lists can be searched
+                with (0, 0);
   slice_grain   loop-3 candidates per slice of a hub (queries of 4+ loops).
 
 The loop order is chosen the same way (``Tuner.tune_order``): the paper's
 plan decision (Sec. 5.3) ranks orders by its cost estimate; here the cost
 model's best few orders are timed on the data at hand and the fastest kept,
 because the estimate does not see list-length skew or the GPU's search paths.
+
+The search starts from the library's own defaults, so what it keeps is never
+slower, as timed, than passing nothing.
 
 Results are cached per (query shape, log2 size bucket, mode) in memory and,
 if a path is given, in a JSON file.  Tuning launches run in count mode; for
@@ -38,6 +42,10 @@ import torch
 from . import Query, choose_shares, plan_cost, run_join
 
 MERGE_OFF = 0xFFFFFFFF
+MERGE_AUTO = (0, 0)
+# counts up when the candidates or the library's defaults change: choices
+# cached before that are timed again
+TRIED = 2
 
 
 @dataclass
@@ -158,7 +166,7 @@ class Tuner:
         """Fastest configuration for this query and data.  mode="materialize"
         (with the output pool size out_capacity, 0 = two-pass) re-chooses the
         merge knobs with materializing launches."""
-        key = shape_key(query, indexes) + f"|P{tuple(P_list)}|min{min_cells}" + (
+        key = shape_key(query, indexes) + f"|P{tuple(P_list)}|min{min_cells}|v{TRIED}" + (
             "" if mode == "count" else f"|{mode}")
         if key in self.cache:
             c = self.cache[key]
@@ -166,7 +174,8 @@ class Tuner:
         stream = stream or torch.cuda.current_stream()
         t0 = time.perf_counter()
         plan = choose_shares(query, indexes, max(P_list))
-        start = Config(shares=plan if math.prod(plan) >= min_cells else [1] * query.n_vars)
+        start = Config(shares=plan if math.prod(plan) >= min_cells else [1] * query.n_vars, item_grain=0,
+                       merge_min=MERGE_AUTO[0], merge_ratio=MERGE_AUTO[1])
         tried = {}
 
         def measure(c: Config) -> float:
@@ -179,8 +188,8 @@ class Tuner:
         best.ms = measure(best)
         knobs = [
             ("shares", share_candidates(query, indexes, P_list, min_cells)),
-            ("item_grain", [16, 64, 256]),
-            ("merge", [(32, 4), (32, 8), (64, 4), (MERGE_OFF, 1)]),
+            ("item_grain", [0, 16, 64, 256]),
+            ("merge", [MERGE_AUTO, (32, 4), (32, 8), (64, 4), (MERGE_OFF, 1)]),
         ]
         if query.n_vars >= 4:
             knobs.append(("slice_grain", [128, 256, 1024]))
@@ -198,7 +207,7 @@ class Tuner:
         if mode == "materialize":
             extra = {"mode": "materialize", "out_capacity": out_capacity}
             best.ms = _time(query, indexes, best, self.reps, stream, **extra)
-            for mm, mr in [(32, 2), (32, 4), (32, 8), (64, 4), (MERGE_OFF, 1)]:
+            for mm, mr in [MERGE_AUTO, (32, 2), (32, 4), (32, 8), (64, 4), (MERGE_OFF, 1)]:
                 c = Config(shares=list(best.shares), item_grain=best.item_grain, merge_min=mm, merge_ratio=mr,
                            slice_grain=best.slice_grain)
                 if c.key() == best.key():
