@@ -300,7 +300,9 @@ typedef struct {
                                   /* for lifted intersections (0: default 16384; at most  */
                                   /* 2^26)                                                 */
     uint64_t out_capacity;        /* materialize: 0 runs a counting pass, then an        */
-                                  /* emitting pass (tuples cell-major, in a fixed order); */
+                                  /* emitting pass (tuples cell-major, in an order fixed */
+                                  /* by the query, the indexes and the other parameters  */
+                                  /* but block_threads, the same on every device);       */
                                   /* > 0 runs one pass writing into an output pool of    */
                                   /* about this many tuples (order not fixed), and falls */
                                   /* back to the emitting pass if the pool overflows     */

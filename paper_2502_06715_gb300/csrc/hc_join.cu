@@ -414,6 +414,13 @@ __host__ __device__ inline uint32_t auto_grain(uint64_t units, uint64_t warps, i
     return (uint32_t)(g < least ? least : g > 64 ? 64 : g);
 }
 
+// The warps auto_grain reckons with where tuples are written: the search
+// kernels' on a whole GB300 (152 SMs of 16 blocks, 12 for 4 loops and more, of
+// 4 warps).  The items' cut decides the order of the tuples, which is promised
+// to be the same whatever the launch: it must not depend on block_threads or
+// on the SMs at hand.
+__host__ __device__ constexpr uint64_t order_warps(int nlev) { return 152u * 4u * (nlev <= 3 ? 16u : 12u); }
+
 // Batch bindings of loops 1..NL-2 (index = loop), one per lane.
 template <int NL, int O>
 struct Frame {
@@ -2303,10 +2310,8 @@ hc_status run_join_impl(const hc_query* q, const hc_index* const* idx, const hc_
     if (cudaMemcpyAsync(&hU, uoff + R->h_ctl.n_entries, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return bail(cuda_fail(cudaGetLastError(), "read units"));
-    // both passes cut the same items: the grain is fixed here
-    const uint32_t grain =
-        qp.grain ? qp.grain
-                 : auto_grain(hU, (uint64_t)gj_grid_any(nv, shape_s, shape_o, false, threads) * (threads / 32), nv);
+    // both passes cut the same items, on every device: the grain is fixed here
+    const uint32_t grain = qp.grain ? qp.grain : auto_grain(hU, order_warps(nv), nv);
     g.grain = grain;
     const uint64_t nitems = (hU + grain - 1) / grain;
     R->n_items = nitems;
