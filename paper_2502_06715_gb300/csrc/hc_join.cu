@@ -62,12 +62,13 @@ struct DPlan {
     int src_f[HC_MAX_VARS][MAXSRC];
     int src_slot[HC_MAX_VARS][MAXSRC];
     // last loop: a parent whose two lists are both >= merge_min long and
-    // within merge_ratio of each other takes the block-merge path (with
-    // merge_auto only where the longer one has no directory); of the others,
-    // one whose shorter list has >= pair_min values is searched by
+    // within merge_ratio of each other takes the block-merge path, if the
+    // longer one is below merge_below or a source of merge_from (4+ loops); of
+    // the others, one whose shorter list has >= pair_min values is searched by
     // the whole warp (probe_pair); the rest are flattened over the lanes
     uint32_t merge_min, merge_ratio, pair_min;
-    int merge_auto;
+    uint32_t merge_below;  // 0xFFFFFFFF: merge whichever list is longer
+    uint32_t merge_from;   // bit q: source q of the last loop is read without a directory
     // searches of runs at least dir_min long go through their bucket
     // directory (0xFFFFFFFF: never)
     uint32_t dir_min;
@@ -448,6 +449,8 @@ struct Acc {
     uint32_t* obuf;   // the warp's staging buffer of OBUF values (materialize), or NULL
     uint64_t* cprof;  // per-cell profile [cells][2] (work units, SM cycles), or NULL
 };
+// A batched query's: its lists merge whichever is longer (batch_create).
+struct BatchAcc : Acc {};
 
 // Output slot of the lane holding rank r among the k = popc(ball) matches
 // of this round (all lanes call).  Two-pass mode: consecutive slots from
@@ -746,8 +749,8 @@ __device__ __forceinline__ void write_tuple(const DPlan& P, uint32_t* o, uint32_
     for (int g = L - 1; g >= 1; --g) o[P.var_of_level[g]] = vals[g];
 }
 
-template <int L, int NL, int S, int O, bool MAT>
-__device__ __forceinline__ void run_level(const DPlan& P, Frame<NL, O>& F, const Entry<NL, S>& E, Acc& A,
+template <int L, int NL, int S, int O, bool MAT, class ACC>
+__device__ __forceinline__ void run_level(const DPlan& P, Frame<NL, O>& F, const Entry<NL, S>& E, ACC& A,
                                           uint32_t nb);
 
 // Last loop, flattened path: count the round's matches, or write them.
@@ -971,8 +974,8 @@ __device__ __forceinline__ void probe_pair(const DPlan& P, const Entry<NL, S>& E
 }
 
 // Compact this round's matches into the batch of loop L and descend.
-template <int L, int NL, int S, int O, bool MAT>
-__device__ __forceinline__ void descend(const DPlan& P, Frame<NL, O>& F, const Entry<NL, S>& E, Acc& A, bool ok,
+template <int L, int NL, int S, int O, bool MAT, class ACC>
+__device__ __forceinline__ void descend(const DPlan& P, Frame<NL, O>& F, const Entry<NL, S>& E, ACC& A, bool ok,
                                         uint32_t v, uint32_t parent, const uint32_t (&nlo)[O],
                                         const uint32_t (&nhi)[O]) {
     const uint32_t ball = __ballot_sync(0xffffffffu, ok);
@@ -994,8 +997,8 @@ __device__ __forceinline__ void descend(const DPlan& P, Frame<NL, O>& F, const E
 // lanes 0..nb-1 (for L == 1 the entry itself, nb == 1, candidates limited to
 // the work item's subrange via E.lo/hi of its shortest list); their
 // candidates are flattened over the lanes, 32 a round.
-template <int L, int NL, int S, int O, bool MAT>
-__device__ __forceinline__ void run_level(const DPlan& P, Frame<NL, O>& F, const Entry<NL, S>& E, Acc& A,
+template <int L, int NL, int S, int O, bool MAT, class ACC>
+__device__ __forceinline__ void run_level(const DPlan& P, Frame<NL, O>& F, const Entry<NL, S>& E, ACC& A,
                                           uint32_t nb) {
     if constexpr (L < NL) {
         const uint32_t lane = lane_id();
@@ -1068,12 +1071,9 @@ __device__ __forceinline__ void run_level(const DPlan& P, Frame<NL, O>& F, const
                     }
                     const uint32_t mn = min(l0, l1), mx = max(l0, l1);
                     merge_class = mn >= P.merge_min && (uint64_t)mx <= (uint64_t)P.merge_ratio * mn;
-                    if (merge_class && P.merge_auto) {
-                        const int qs = l0 > l1 ? qa : qb;  // the longer list, which would be searched
-                        const DAtom& ds = P.atom[P.src_atom[L][qs]];
+                    if constexpr (NL >= 4 && std::is_same_v<ACC, Acc>)
                         merge_class =
-                            qs == lift_q || mx < P.dir_min || (P.src_top[L][qs] ? ds.g1 : ds.g2) == nullptr;
-                    }
+                            merge_class && (mx < P.merge_below || (P.merge_from >> (l0 > l1 ? qa : qb) & 1u));
                     pair_class = !merge_class && mn >= P.pair_min;
                 }
             }
@@ -1190,8 +1190,8 @@ __device__ __forceinline__ void run_level(const DPlan& P, Frame<NL, O>& F, const
 // all entries' units (a unit is a loop-2 candidate, or a slice of one for
 // deep queries).  Returns the item's count; cell counts are added when
 // requested.  elo/ehi are the warp's shared-memory rows for entry ranges.
-template <int NL, int S, int O, bool MAT>
-__device__ __forceinline__ uint64_t search_item(const DPlan& P, Frame<NL, O>& F, Acc& A, uint32_t (*elo)[S],
+template <int NL, int S, int O, bool MAT, class ACC>
+__device__ __forceinline__ uint64_t search_item(const DPlan& P, Frame<NL, O>& F, ACC& A, uint32_t (*elo)[S],
                                                 uint32_t (*ehi)[S], uint64_t item, uint32_t grain, uint32_t E_n,
                                                 uint64_t U, const uint32_t* __restrict__ e_cell,
                                                 const uint32_t* __restrict__ e_x, const uint32_t* __restrict__ e_rng,
@@ -1422,7 +1422,7 @@ __global__ void __launch_bounds__(128, ((NLA <= 3 && NLB <= 3) ? 16 : 12))
     if (dev_err_set(&qs[0].ctl->err)) return;  // the item-offset scan gave up a wait
     const uint64_t total_items = item_off[n];
     uint32_t cur = 0xFFFFFFFFu;
-    Acc A;
+    BatchAcc A;
     A.count = 0;
     A.work = 0;
     A.out_pos = 0;
@@ -1495,7 +1495,7 @@ __global__ void __launch_bounds__(128, 12)
     if (dev_err_set(&qs[0].ctl->err)) return;  // the item-offset scan gave up a wait
     const uint64_t total_items = item_off[n];
     uint32_t cur = 0xFFFFFFFFu;
-    Acc A;
+    BatchAcc A;
     A.count = 0;
     A.work = 0;
     A.out_pos = 0;
@@ -2030,7 +2030,13 @@ hc_status plan_query(const hc_query* q, const hc_index* const* idx, const hc_joi
     // (the arena of lifted lists, or directories switched off).  Merging every
     // pair of length ratio <= 4, the triangle on R-MAT 22 in 64 cells took
     // 75.1 ms; searched through the directories it takes 54.0 ms.
-    P.merge_auto = prm->merge_min == 0 && prm->merge_ratio == 0;
+    // Which sources those are is settled here, and up to 3 loops, whose lists
+    // are lifted nowhere, whether there are any: without them nothing is
+    // merged, with them (a top-level list in the last loop) every pair may be.
+    // Read from the atoms by every warp instead, it cost the searches 1.2 %
+    // (triangles of R-MAT 19, merging off, 10.25 ms against 10.14), and as a
+    // plan constant still 0.6 % at 3 loops (10.21).
+    const bool merge_auto = prm->merge_min == 0 && prm->merge_ratio == 0;
     P.merge_min = prm->merge_min ? prm->merge_min : 32;
     P.pair_min = prm->pair_min ? prm->pair_min : 32;
     P.merge_ratio = prm->merge_ratio ? prm->merge_ratio : 4;
@@ -2060,6 +2066,15 @@ hc_status plan_query(const hc_query* q, const hc_index* const* idx, const hc_joi
             P.far_mask = 0;
         }
     }
+    P.merge_below = merge_auto ? P.dir_min : 0xFFFFFFFFu;
+    P.merge_from = 0;
+    for (int qq = 0; qq < P.nsrc[nv - 1]; ++qq) {
+        const DAtom& a = P.atom[P.src_atom[nv - 1][qq]];
+        // a lifted list pairs with the one other list left of three or more
+        const bool lifted = P.lift && qq == P.far0 && P.nsrc[nv - 1] > 2;
+        if (lifted || (P.src_top[nv - 1][qq] ? a.g1 : a.g2) == nullptr) P.merge_from |= 1u << qq;
+    }
+    if (nv <= 3 && merge_auto && P.merge_from == 0 && P.dir_min <= P.merge_min) P.merge_min = 0xFFFFFFFFu;
     // loop-1 candidates are bounded by any loop-1 atom's rows times the
     // number of cells that read each of its partitions
     uint64_t cand_bound = UINT64_MAX;
@@ -2585,8 +2600,10 @@ hc_status batch_create(const hc_query* qs, const hc_index* const* idx_flat, cons
         hc_status st = plan_query(&qs[i], idx_flat + off, &prm[i], s, &B->plans[i]);
         if (st != HC_OK) return bail(st);
         // the batched kernels, at 40 registers for two shapes, search slower
-        // than they merge: 96 queries of 30,000 edges, 18.6 against 19.1 ms
-        B->plans[i].P.merge_auto = 0;
+        // than they merge, so the automatic rule is not theirs: five kinds of
+        // batch, 24 to 96 queries of 1,500 to 60,000 edges, take as long or up
+        // to 5 % longer with it (96 of 30,000: 13.57 against 13.07 ms)
+        B->plans[i].P.merge_min = prm[i].merge_min ? prm[i].merge_min : 32;
         if (B->plans[i].P.lift) B->arena_stride = std::max(B->arena_stride, B->plans[i].P.arena_words);
         off += qs[i].n_atoms;
         const int c = shape_class(B->plans[i]);
