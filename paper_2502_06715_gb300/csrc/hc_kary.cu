@@ -752,6 +752,7 @@ constexpr uint32_t KPAIR_MIN = 32;  // default per-binding threshold of the last
 // by binary search.  KP_POS: a top level's position map.
 constexpr uint32_t KP_BIT = 0x800u, KP_DIRECT = 0x200u, KP_DIR = 0x100u, KP_POS = 0x400u;
 constexpr uint32_t KDENSE_WORDS = 512;  // the word path of the last loop: words one lane takes, at most
+constexpr uint32_t KDENSE_TURN = 4;     // fixed cost of a parent whose words the warp shares, in words
 constexpr int KJ_MAXT = 128;      // threads per block of the search kernel, at most
 constexpr int KJ_WARPS = KJ_MAXT / 32;
 
@@ -1026,21 +1027,23 @@ __device__ __forceinline__ void krange(const KPlan& P, const KWarp<NV>& S, int L
     hi = S.rhi[f - 1][r][a];
 }
 
-// Last loop, counting: parent b's result when all its lists are dense, each
-// kept as a bitmap (dense_of): the popcount of the words' AND over the values
-// they all span, a word for 32 values, one parent a lane.  Returns false when
-// a list is not dense, or the words are too many for one lane or not fewer
-// than the parent's c candidates.  LW on boxes of about 256 a side: the
-// search took 6.65 ms with a 4-byte read per value and list, 1.3 ms so.
+// Last loop, counting: a parent whose lists are all dense, each kept as a
+// bitmap (dense_of), has the popcount of the words' AND over the values that
+// they all span, a word for 32 values.
+struct KDense {
+    const uint32_t* p[KMAXS];  // list q's word of the values 32 i .. 32 i + 31 is p[q][i]
+    uint32_t i0, words;        // the words all lists span: [i0, i0 + words)
+};
+
+// Parent b's words; false when a list is not dense.
 template <int NV>
-__device__ __forceinline__ bool kdense(const KPlan& P, const KWarp<NV>& S, uint32_t b, uint32_t c, uint32_t& n) {
+__device__ __forceinline__ bool kdense_init(const KPlan& P, const KWarp<NV>& S, uint32_t b, KDense& K) {
     constexpr int L = NV - 1;
     const int ns = P.nsrc[L];
     uint32_t lo = 0, hi = 0xFFFFFFFFu;
-    const uint32_t* p[KMAXS];
 #pragma unroll
     for (int q = 0; q < KMAXS; ++q) {
-        p[q] = nullptr;
+        K.p[q] = nullptr;
         if (q < ns) {
             const KSrc& s = P.src[L][q];
             uint32_t r0, r1;
@@ -1049,23 +1052,27 @@ __device__ __forceinline__ bool kdense(const KPlan& P, const KWarp<NV>& S, uint3
             const uint32_t vmin = __ldg(s.v + r0), vmax = __ldg(s.v + r1 - 1);
             const Dense D = dense_of(r0, r1, vmin, vmax);
             if (!D.ok) return false;
-            p[q] = s.b + D.w0 - (D.vbase >> 5);  // the word of values 32 i .. 32 i + 31 is p[q][i]
+            K.p[q] = s.b + D.w0 - (D.vbase >> 5);
             lo = max(lo, D.vbase);
             hi = min(hi, vmax);
         }
     }
-    const uint32_t i0 = lo >> 5, i1 = hi >> 5;
-    const uint32_t words = hi >= lo ? i1 - i0 + 1u : 0u;
-    if (words > KDENSE_WORDS || words >= c) return false;
-    n = 0;
-    for (uint32_t i = i0; i < i0 + words; ++i) {
-        uint32_t w = __ldg(p[0] + i);
+    K.i0 = lo >> 5;
+    K.words = hi >= lo ? (hi >> 5) - K.i0 + 1u : 0u;
+    return true;
+}
+
+// The bits set in all lists, over the words first, first + step, ...
+__device__ __forceinline__ uint32_t kdense_count(const KDense& K, int ns, uint32_t first, uint32_t step) {
+    uint32_t n = 0;
+    for (uint32_t i = K.i0 + first; i < K.i0 + K.words; i += step) {
+        uint32_t w = __ldg(K.p[0] + i);
 #pragma unroll
         for (int q = 1; q < KMAXS; ++q)
-            if (q < ns) w &= __ldg(p[q] + i);
+            if (q < ns) w &= __ldg(K.p[q] + i);
         n += __popc(w);
     }
-    return true;
+    return n;
 }
 
 // Start loop L with parents 0..nb-1: each parent's shortest list and the
@@ -1098,13 +1105,20 @@ __device__ __forceinline__ void kinit_level(const KPlan& P, KWarp<NV>& S, int L,
         }
     }
     // last loop, counting: a parent whose lists are all dense is done by its
-    // lane, word by word; of the others, one with many candidates leaves the
-    // flattened rounds for the per-binding path (kpair)
+    // lane, word by word (LW on boxes of about 256 a side: the search took
+    // 6.65 ms with a 4-byte read per value and list, 1.33 ms so); of the others,
+    // one with many candidates leaves the flattened rounds for the per-binding
+    // path (kpair).  So does one that is long where there are few, as a lane
+    // would walk its words while the others wait: at 32 candidates a word,
+    // longer than nb turns of 1/32 of it and KDENSE_TURN words (LW on a box of
+    // 16 x 16 x 16 x 8000: 0.25 ms on lanes, 0.07 ms in turns)
     bool lng = false;
     if (!MAT && L == NV - 1 && L > 1 && P.last_dense && lane < nb && c >= DIR_MIN) {
-        uint32_t n;
-        if (kdense<NV>(P, S, lane, (uint32_t)c, n)) {
-            cnt += n;
+        const uint32_t c32 = (uint32_t)c;
+        KDense K;
+        if ((c32 < P.pair_min || c32 <= nb * (c32 / 32 + 32 * KDENSE_TURN)) && kdense_init<NV>(P, S, lane, K) &&
+            K.words <= KDENSE_WORDS) {
+            cnt += kdense_count(K, P.nsrc[L], 0, 1);
             c = 0;
         }
     }
@@ -1130,7 +1144,8 @@ __device__ __forceinline__ void kinit_level(const KPlan& P, KWarp<NV>& S, int L,
     __syncwarp();
 }
 
-// The per-binding path of the last loop: parent b's candidates, the
+// The per-binding path of the last loop: counting, the words of the lists'
+// AND where all are dense, 32 at a time; else parent b's candidates, the
 // elements of its shortest list, 128 per iteration (lane l takes the
 // elements l, l + 32, l + 64, l + 96 of each block), searched in each other
 // list in turn with the four reads of a lane issued together.  A list's
@@ -1149,6 +1164,13 @@ __device__ __forceinline__ void kpair(const KPlan& P, KWarp<NV>& S, uint32_t b, 
     if (ns == 1 && !MAT) {  // nothing to search: every candidate is a result
         if (lane == 0) cnt += a1 - a0;
         return;
+    }
+    if (!MAT && P.last_dense) {  // all lists dense: the words of their AND, spread over the lanes
+        KDense K;
+        if (kdense_init<NV>(P, S, b, K)) {
+            cnt += kdense_count(K, ns, lane, 32);
+            return;
+        }
     }
     // lane q sets up list q once for the whole parent
     __syncwarp();
@@ -1419,7 +1441,7 @@ __global__ void __launch_bounds__(KJ_MAXT) kjoin_kernel(const KPlan* __restrict_
     KWarp<NV>& S = WS[w];
     if (dev_err_set(&ctl->err)) return;  // the unit-offset scan gave up a wait
     if (threadIdx.x == 0) {  // levels without dense runs: their bitmaps are not looked at
-        int all = 1;
+        int all = P.nsrc[NV - 1] > 1;  // a single list has nothing to intersect
         for (int q = 0; q < P.nsrc[NV - 1]; ++q) {
             KSrc& s = P.src[NV - 1][q];
             if (s.b != nullptr && __ldg(s.b) == 0) s.b = nullptr;
