@@ -279,6 +279,12 @@ hc_status hc_plan_cost(const hc_query* q, const hc_index* const* idx, const uint
  * device scratch per resident warp, and is off with HC_FLAG_STATS (the work
  * counter measures the unrewritten loops) or with: */
 #define HC_FLAG_NO_LIFT 8u
+/* Testing only: the first tile of the loop-1 pass never publishes its
+ * look-back status, so the tiles after it wait until the limit
+ * (hc_set_wait_limit_ns) and the call, or hc_batch_counts of its batch,
+ * returns HC_ERR_TIMEOUT (loop 1 must span more than one tile: 256 values of
+ * its shortest lists). */
+#define HC_FLAG_TEST_STALL_LOOP1 0x100u
 
 typedef struct {
     uint32_t shares[HC_MAX_VARS]; /* P_v per variable id (>= 1); their product = cells  */

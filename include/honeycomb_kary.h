@@ -38,7 +38,10 @@ typedef struct hc_kindex hc_kindex;
  *               of 0..k-1 (NULL: 0, 1, ..).
  *   flags       HC_BUILD_CHECK_DUPLICATES: a repeated row returns
  *               HC_ERR_DUPLICATE instead of an index; HC_BUILD_TIME_KERNELS:
- *               the sort and the level scan are timed (hc_kindex_view).
+ *               the sort and the level scan are timed (hc_kindex_view);
+ *               HC_BUILD_TEST_STALL_SORT (testing only, as hc_build_index):
+ *               the first tile of the packed keys' first radix pass, or of
+ *               the last level's but one, never publishes its status.
  * The rows are sorted as one 64-bit key per row when the levels' value bits
  * add up to at most 64 (packed), else one level at a time (stable by
  * position).  Waits for the GPU (column maxima, level sizes).  Rows must be

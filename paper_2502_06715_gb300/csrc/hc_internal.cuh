@@ -438,9 +438,10 @@ hc_status build_index_impl(const uint32_t* d_pairs, uint64_t n, uint32_t attr_or
 // d_pairs sorted by (first, second) into keys (first << 32 | second, [n]
 // allocated here), the largest values being known; enqueued without waiting.
 // A look-back that gives up sets DEV_ERR_TIMEOUT in *d_err, after which the
-// keys are not valid.
+// keys are not valid.  `withhold` (testing only) makes the first pass's waits
+// run out.
 hc_status sort_pairs(const uint2* d_pairs, uint64_t n, uint32_t max_first, uint32_t max_second, uint32_t* d_err,
-                     cudaStream_t s, uint64_t** out_keys);
+                     cudaStream_t s, uint64_t** out_keys, bool withhold = false);
 hc_status partition_impl(const hc_index* idx, uint32_t seed_a, uint32_t pa, uint32_t seed_b,
                          uint32_t pb, cudaStream_t s, hc_partitioned** out);
 void partitioned_release(hc_partitioned* p, cudaStream_t s);

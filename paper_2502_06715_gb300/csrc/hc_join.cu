@@ -151,7 +151,8 @@ struct L0Job {
     JoinCtl* ctl;
     uint64_t* status;  // look-back words: [tiles] entry counts, then [tiles] work units
     uint32_t tiles;
-    uint32_t tile0;  // batched: the query's first tile
+    uint32_t tile0;     // batched: the query's first tile
+    uint32_t withhold;  // testing only: tile 0 never publishes, so that the waits on it run out
 };
 
 // A tile of loop 1: thread t's candidate is value t of the concatenation of
@@ -293,7 +294,7 @@ __device__ __forceinline__ bool l0_tile(const DPlan& P, const L0Job& J, uint32_t
     if (w < 2) {  // warp 0: entries, warp 1: units
         const uint64_t tot = warp_sum64(lane < L0_WARPS ? (w == 0 ? (uint64_t)sh.wcnt[lane] : sh.wunits[lane]) : 0);
         uint64_t* st = J.status + (uint64_t)w * J.tiles;
-        if (lane == 0) st_relaxed(st + tile, (tile == 0 ? LB_INC : LB_AGG) | tot);
+        if (lane == 0 && !(J.withhold && tile == 0)) st_relaxed(st + tile, (tile == 0 ? LB_INC : LB_AGG) | tot);
         uint64_t excl = 0;
         if (tile != 0) {
             excl = warp_lookback(st, tile, &J.ctl->err, wait_ns);
@@ -1841,6 +1842,7 @@ hc_status result_get(hc_result* R, hc_result_view* v) {
 struct QueryPlan {
     DPlan P;
     int nv = 0, shape_s = 2, shape_o = 2, threads = 128, stats = 0;
+    bool stall = false;  // HC_FLAG_TEST_STALL_LOOP1
     uint32_t grain = 0;  // work units per item (0: auto_grain)
     uint64_t ncells = 1, cand_bound = 1;
     std::vector<hc_partitioned*> parts;
@@ -1903,6 +1905,7 @@ hc_status plan_query(const hc_query* q, const hc_index* const* idx, const hc_joi
     out->nv = nv;
     out->ncells = ncells;
     out->stats = (prm->flags & (HC_FLAG_STATS | HC_FLAG_CELL_PROFILE)) ? 1 : 0;
+    out->stall = (prm->flags & HC_FLAG_TEST_STALL_LOOP1) != 0;
 
     DPlan& P = out->P;
     memset(&P, 0, sizeof(P));
@@ -2133,7 +2136,8 @@ hc_status alloc_level1_cells(uint64_t ncells, Alloc& a, Level1* L) {
 // The query's loop-1 job.  With one cell the candidates are known here: the
 // shortest of the whole top-level lists.
 static L0Job l0_job(const QueryPlan& qp, const Level1& L, JoinCtl* ctl, uint64_t* status) {
-    L0Job J{L.d_plan, nullptr, qp.cand_bound, L.e_cell, L.e_x, L.e_rng, L.e_split, L.uoff, ctl, status, l0_tiles(qp), 0};
+    L0Job J{L.d_plan, nullptr, qp.cand_bound, L.e_cell, L.e_x, L.e_rng, L.e_split, L.uoff, ctl, status, l0_tiles(qp), 0,
+            qp.stall ? 1u : 0u};
     if (qp.ncells > 1) {
         J.candoff = L.candoff;
     } else {

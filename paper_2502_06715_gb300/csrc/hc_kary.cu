@@ -571,6 +571,7 @@ hc_status build_kindex_impl(const uint32_t* d_rows, uint64_t n, uint32_t k, cons
     const uint32_t pid_bits = bit_width((uint32_t)(np - 1));
 
     const bool timed = (flags & HC_BUILD_TIME_KERNELS) != 0;
+    const bool stall = (flags & HC_BUILD_TEST_STALL_SORT) != 0;
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
     auto destroy_events = [&]() {
         for (auto& e : ev)
@@ -610,7 +611,7 @@ hc_status build_kindex_impl(const uint32_t* d_rows, uint64_t n, uint32_t k, cons
         const uint32_t kb = total_bits + pid_bits;  // the packed key's bits, above and below bit 32
         const uint32_t hi = kb > 32 ? (uint32_t)((1ull << (kb - 32)) - 1) : 0u;
         const uint32_t lo = kb >= 32 ? 0xFFFFFFFFu : (uint32_t)((1ull << kb) - 1);
-        if ((st = sort_pairs(pk, n, hi, lo, &ctl->err, s, &keys)) != HC_OK) return bail2(st);
+        if ((st = sort_pairs(pk, n, hi, lo, &ctl->err, s, &keys, stall)) != HC_OK) return bail2(st);
         src.keys = keys;
     } else {
         uint2* pairs;
@@ -626,7 +627,9 @@ hc_status build_kindex_impl(const uint32_t* d_rows, uint64_t n, uint32_t k, cons
                 kpid_pairs_kernel<<<grid_of(n, 256, 8), 256, 0, s>>>(d_rows, n, L, Pt, cur, pairs, &ctl->err);
             if (cudaError_t le = launch_check()) return bail2(cuda_fail(le, "kperm_pairs_kernel"));
             const uint32_t top = d >= 0 ? x->maxv[d] : (uint32_t)(np - 1);
-            if ((st = sort_pairs(pairs, n, top, (uint32_t)(n - 1), &ctl->err, s, &keys)) != HC_OK) return bail2(st);
+            // testing only: a sort has run before the one that stalls, and others follow
+            const bool hold = stall && d == (int)k - 2;
+            if ((st = sort_pairs(pairs, n, top, (uint32_t)(n - 1), &ctl->err, s, &keys, hold)) != HC_OK) return bail2(st);
             uint32_t* nxt = cur == pa ? pb : pa;
             kperm_compose_kernel<<<grid_of(n, 256, 8), 256, 0, s>>>(keys, cur, nxt, n, &ctl->err);
             if (cudaError_t le = launch_check()) return bail2(cuda_fail(le, "kperm_compose_kernel"));

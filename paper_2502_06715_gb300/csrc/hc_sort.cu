@@ -978,7 +978,7 @@ hc_status build_index_impl(const uint32_t* d_pairs, uint64_t n, uint32_t ao, uin
 }
 
 hc_status sort_pairs(const uint2* d_pairs, uint64_t n, uint32_t max_first, uint32_t max_second, uint32_t* d_err,
-                     cudaStream_t s, uint64_t** out_keys) {
+                     cudaStream_t s, uint64_t** out_keys, bool withhold) {
     *out_keys = nullptr;
     void* p;
     HC_TRY(dev_alloc(&p, std::max<uint64_t>(n, 1) * 8, s));
@@ -995,7 +995,7 @@ hc_status sort_pairs(const uint2* d_pairs, uint64_t n, uint32_t max_first, uint3
             if (cudaMemsetAsync(counters, 0, MAX_PASSES * sizeof(uint32_t), s) != cudaSuccess)
                 st = cuda_fail(cudaGetLastError(), "memset");
             else
-                st = radix_passes(d_pairs, true, 0, n, specs, keys, tmp, counters, d_err, s);
+                st = radix_passes(d_pairs, true, 0, n, specs, keys, tmp, counters, d_err, s, nullptr, withhold);
         }
     }
     if (st != HC_OK) {

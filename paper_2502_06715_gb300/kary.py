@@ -137,12 +137,13 @@ class KIndex:
 
 def build_kindex(rows: torch.Tensor, level_cols: Sequence[int] | None = None, check_duplicates: bool = False,
                  stream=None, time_kernels: bool = False, seeds: Sequence[int] | None = None,
-                 shares: Sequence[int] | None = None) -> KIndex:
+                 shares: Sequence[int] | None = None, test_stall: bool = False) -> KIndex:
     """k-level CoCo of a relation given as an (n, k) 32-bit CUDA tensor, k = 1..3,
     with level d holding column level_cols[d] (default 0, 1, ..).  With
     ``shares`` (and ``seeds``), one per column, the relation is partitioned
     for HyperCube shares first (Sec. 4) and each partition gets its own
-    trie."""
+    trie.  ``test_stall`` is for testing the bounded-wait error path only: the
+    first tile of a sort pass never publishes its status."""
     if not isinstance(rows, torch.Tensor) or not rows.is_cuda or rows.dim() != 2 or rows.element_size() != 4:
         raise TypeError("rows must be an (n, k) 32-bit CUDA tensor")
     r = rows.contiguous()
@@ -151,7 +152,8 @@ def build_kindex(rows: torch.Tensor, level_cols: Sequence[int] | None = None, ch
     if level_cols is not None:
         cols = (ctypes.c_uint8 * _lib.HC_KMAX_ARITY)(*([int(c) for c in level_cols] + [0] * (3 - len(level_cols))))
     flags = (_lib.HC_BUILD_CHECK_DUPLICATES if check_duplicates else 0) | (
-        _lib.HC_BUILD_TIME_KERNELS if time_kernels else 0)
+        _lib.HC_BUILD_TIME_KERNELS if time_kernels else 0) | (
+        _lib.HC_BUILD_TEST_STALL_SORT if test_stall else 0)
     out = ctypes.c_void_p()
     ptr = ctypes.c_void_p(r.data_ptr() if r.numel() else 0)
     if shares is None:
