@@ -285,6 +285,9 @@ hc_status hc_plan_cost(const hc_query* q, const hc_index* const* idx, const uint
  * returns HC_ERR_TIMEOUT (loop 1 must span more than one tile: 256 values of
  * its shortest lists). */
 #define HC_FLAG_TEST_STALL_LOOP1 0x100u
+/* Testing only, likewise: the first tile of the first radix pass of every
+ * partitioned copy that the call makes (indexes of more than 6,144 rows). */
+#define HC_FLAG_TEST_STALL_PARTITION 0x200u
 
 typedef struct {
     uint32_t shares[HC_MAX_VARS]; /* P_v per variable id (>= 1); their product = cells  */

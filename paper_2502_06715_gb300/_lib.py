@@ -28,6 +28,7 @@ HC_BUILD_TIME_KERNELS = 2
 HC_BUILD_TEST_STALL_SORT = 0x100
 HC_BUILD_TEST_STALL_SCAN = 0x200
 HC_FLAG_TEST_STALL_LOOP1 = 0x100
+HC_FLAG_TEST_STALL_PARTITION = 0x200
 
 STATUS = {0: "HC_OK", 1: "HC_ERR_ARG", 2: "HC_ERR_OOM", 3: "HC_ERR_CUDA", 4: "HC_ERR_TIMEOUT",
           5: "HC_ERR_CAPACITY", 6: "HC_ERR_DUPLICATE", 7: "HC_ERR_BUSY"}

@@ -443,7 +443,7 @@ hc_status build_index_impl(const uint32_t* d_pairs, uint64_t n, uint32_t attr_or
 hc_status sort_pairs(const uint2* d_pairs, uint64_t n, uint32_t max_first, uint32_t max_second, uint32_t* d_err,
                      cudaStream_t s, uint64_t** out_keys, bool withhold = false);
 hc_status partition_impl(const hc_index* idx, uint32_t seed_a, uint32_t pa, uint32_t seed_b,
-                         uint32_t pb, cudaStream_t s, hc_partitioned** out);
+                         uint32_t pb, cudaStream_t s, hc_partitioned** out, bool withhold = false);
 void partitioned_release(hc_partitioned* p, cudaStream_t s);
 void index_release(hc_index* idx, cudaStream_t s);
 hc_status build_unary_impl(const uint32_t* d_values, uint64_t n, uint32_t max_value, cudaStream_t s,
@@ -466,6 +466,7 @@ hc_status exclusive_scan_u32_to_u64(const uint32_t* d_in, uint64_t* d_out, uint6
 hc_status exclusive_scan_u64(const uint64_t* d_in, uint64_t* d_out, uint64_t n_max, const uint32_t* d_n,
                              uint32_t* d_err, cudaStream_t s);
 hc_status partitioned_sync(hc_partitioned* p);
+const uint32_t* partitioned_err_ptr(const hc_partitioned* p);  // device; nonzero: the copy is not valid
 void result_release(hc_result* r);
 // Record the event that opens (end = false) or closes timed search launch
 // R->n_timed on s, creating it first; closing advances n_timed.

@@ -117,11 +117,25 @@ __device__ __forceinline__ void top_range(const DAtom& a, uint32_t cell, uint32_
 }
 
 // ------------------------------------------------------------------ loop 1
-// Per cell: length of the shortest top-level list of loop 1.
+// The error words of a query's partitioned copies.
+struct PartErrs {
+    const uint32_t* err[HC_MAX_ATOMS];
+    int n;
+};
+
+// Per cell: length of the shortest top-level list of loop 1.  A copy whose
+// partitioning gave up a wait has no levels to read: its error becomes the
+// join's, so that this kernel and all after it read nothing.
 __global__ void l0_count_kernel(const DPlan* __restrict__ gP, uint32_t* __restrict__ cand, JoinCtl* ctl, int stats,
-                                uint64_t* __restrict__ cprof) {
+                                uint64_t* __restrict__ cprof, const __grid_constant__ PartErrs parts) {
     __shared__ DPlan P;
     load_plan(P, gP);
+    bool failed = false;
+    for (int k = 0; k < parts.n; ++k) failed = failed || dev_err_set(parts.err[k]);
+    if (failed) {
+        if (threadIdx.x == 0) atomicOr(&ctl->err, DEV_ERR_TIMEOUT);
+        return;
+    }
     uint64_t work = 0;
     for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < P.ncells; c += gridDim.x * blockDim.x) {
         uint32_t m = 0xFFFFFFFFu;
@@ -1847,6 +1861,7 @@ struct QueryPlan {
     uint64_t ncells = 1, cand_bound = 1;
     std::vector<hc_partitioned*> parts;
     std::vector<const hc_index*> part_src;  // the index each partitioned copy was made from
+    PartErrs part_errs{};                   // and their error words
 };
 
 static void release_parts(std::vector<hc_partitioned*>& parts, cudaStream_t s) {
@@ -1967,10 +1982,12 @@ hc_status plan_query(const hc_query* q, const hc_index* const* idx, const hc_joi
                     part = c;
             }
             if (!part) {
-                const hc_status st = partition_impl(ix, seed_a, pa, seed_b, pb, s, &part);
+                const hc_status st = partition_impl(ix, seed_a, pa, seed_b, pb, s, &part,
+                                                    (prm->flags & HC_FLAG_TEST_STALL_PARTITION) != 0);
                 if (st != HC_OK) return bail(st);
                 out->parts.push_back(part);
                 out->part_src.push_back(ix);
+                out->part_errs.err[out->part_errs.n++] = partitioned_err_ptr(part);
             }
             d.v1 = part->d_v1;
             d.o1 = part->d_o1;
@@ -2152,7 +2169,8 @@ hc_status enqueue_cells(const QueryPlan& qp, const Level1& L, JoinCtl* ctl, cuda
     const int tpb = 256;
     const uint64_t ncells = qp.ncells;
     l0_count_kernel<<<(unsigned)std::min<uint64_t>((ncells + tpb - 1) / tpb, 4096), tpb, 0, s>>>(L.d_plan, L.cand, ctl,
-                                                                                                 qp.stats, cell_prof);
+                                                                                                 qp.stats, cell_prof,
+                                                                                                 qp.part_errs);
     if (cudaError_t le = launch_check()) return cuda_fail(le, "l0_count_kernel");
     return exclusive_scan_u32_to_u64(L.cand, L.candoff, ncells, nullptr, &ctl->err, s);
 }

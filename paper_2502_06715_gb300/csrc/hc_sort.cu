@@ -1081,7 +1081,7 @@ void partitioned_release(hc_partitioned* p, cudaStream_t s) {
 }
 
 hc_status partition_impl(const hc_index* idx, uint32_t seed_a, uint32_t pa, uint32_t seed_b, uint32_t pb,
-                         cudaStream_t s, hc_partitioned** out) {
+                         cudaStream_t s, hc_partitioned** out, bool withhold) {
     if (!out) return fail(HC_ERR_ARG, "partition: out is NULL");
     *out = nullptr;
     if (!idx) return fail(HC_ERR_ARG, "partition: index is NULL");
@@ -1132,7 +1132,7 @@ hc_status partition_impl(const hc_index* idx, uint32_t seed_a, uint32_t pa, uint
             std::vector<DigitSpec> specs;
             for (uint32_t b = 0; b < bits_of(np - 1); b += 8) specs.push_back({1, b, seed_a, pa, seed_b, pb});
             if ((st = radix_passes(idx->d_keys, false, 0, n, specs, part->d_keys, tmp, d_ctl->tile_counter,
-                                   &d_ctl->err, s)) != HC_OK)
+                                   &d_ctl->err, s, nullptr, withhold)) != HC_OK)
                 return bail(st);
         }
         if ((st = run_boundary(part->d_keys, n, true, seed_a, pa, seed_b, pb, part->d_v1, part->d_o1, part->d_v2, tmp,

@@ -128,3 +128,24 @@ def test_kary_build(hc, wide, shares, limit_ns):
     else:
         got = hc.run_kjoin(hc.KQuery(3, ((0, 1, 2),)), [hc.build_kindex(d)]).count
         assert got == rows.shape[0]
+
+
+@pytest.mark.parametrize("shares", [[4, 1, 1], [3, 2, 2], [40, 20, 1]])
+def test_partitioned_copies(hc, graph, shares):
+    """A partitioned copy whose sort gave up has no levels: the join that made
+    it must not read them (one and two radix passes, one and three copies)."""
+    import torch
+
+    ix, want, _ = graph
+    flag = hc._lib.HC_FLAG_TEST_STALL_PARTITION
+    with times_out(hc, 20_000_000):
+        hc.run_join_async(hc.TRIANGLE, [ix] * 3, shares=shares, flags=flag).count()
+    out = torch.empty((want, 3), dtype=torch.int32)
+    with times_out(hc, 20_000_000):
+        hc.run_join_to_host(hc.TRIANGLE, [ix] * 3, out, shares=shares, flags=flag)
+    side = torch.cuda.Stream()
+    with times_out(hc, 20_000_000):
+        bad = hc.Batch([hc.TRIANGLE] * 2, [[ix] * 3] * 2, [{}, {"shares": shares, "flags": flag}], stream=side)
+        bad.launch(side)
+        bad.counts()
+    assert hc.run_join(hc.TRIANGLE, [ix] * 3, shares=shares).count == want
