@@ -237,9 +237,16 @@ def source_hash(sources) -> str:
     return h.hexdigest()
 
 
-def profiled_traffic(note: str = None, sources=("hc_join.cu", "hc_internal.cuh")):
+def schedule_name(shares, item_grain, merge_min, merge_ratio) -> str:
+    """A search's cells and schedule, as the committed ncu summaries name them."""
+    merge = "off" if merge_min == 0xFFFFFFFF else f"{merge_min},{merge_ratio}" if merge_min or merge_ratio else "auto"
+    return f"shares {'x'.join(str(s) for s in shares)}, item grain {item_grain or 'by size'}, merge {merge}"
+
+
+def profiled_traffic(note: str = None, sources=("hc_join.cu", "hc_internal.cuh"), schedule: str = None):
     """Per-launch DRAM bytes of a kernel from a committed ncu summary, if it
-    was taken on the current source of the files that hold the kernel."""
+    was taken on the current source of the files that hold the kernel and,
+    where the bytes depend on it, under the same cells and schedule."""
     try:
         text = open(note or PROFILE_NOTE).read()
     except OSError:
@@ -250,6 +257,10 @@ def profiled_traffic(note: str = None, sources=("hc_join.cu", "hc_internal.cuh")
         return None
     if source_hash(sources) != h.group(1):
         return None
+    if schedule is not None:
+        taken = re.search(r"^\s*schedule: (.+?)\s*$", text, re.M)
+        if not taken or taken.group(1) != schedule:
+            return None
     return int(m.group(1))
 
 
@@ -390,7 +401,9 @@ def main():
     achieved = alg_bytes / avg_launch_s / 1e9 if avg_launch_s > 0 else 0.0
     roofline = {"bound": "hbm", "kernel": "gj_kernel (persistent search)", "achieved": round(achieved, 1),
                 "peak": peak, "peak_kind": peak_kind, "unit": "GB/s", "frac": round(achieved / peak, 4),
-                "traffic": profiled_traffic(), "alg_bytes_per_launch": alg_bytes,
+                "traffic": profiled_traffic(schedule=schedule_name(shares, a.grain, knobs.get("merge_min", 0),
+                                                                   knobs.get("merge_ratio", 0))),
+                "alg_bytes_per_launch": alg_bytes,
                 "avg_launch_ms": round(avg_launch_s * 1e3, 3)}
 
     e2e = None
@@ -584,7 +597,8 @@ def other_workload(a, world, rank, local):
     tune_s = time.perf_counter() - t
     sep_counts = [hc.run_join(q, l, **o).count for q, l, o in zip(qs, idx, opts)]
     side = torch.cuda.Stream(dev)
-    b = hc.Batch(qs, idx, opts, stream=side)
+    # a batch cuts its items over all its queries and merges by its own rule
+    b = hc.Batch(qs, idx, [{k: o[k] for k in ("shares", "slice_grain")} for o in opts], stream=side)
     l0 = hc.kernel_launches()
     b.capture(side)
     per_replay = hc.kernel_launches() - l0  # kernels recorded in the graph
@@ -728,7 +742,7 @@ def skew_workload(a, world, rank, local):
     d = torch.from_numpy(ep.view(np.int32)).to(dev)
     ix = hc.build_index(d, 0)
     q = hc.TRIANGLE
-    knobs = {"item_grain": a.grain or 64, "merge_min": 0xFFFFFFFF, "merge_ratio": 1}
+    knobs = {"item_grain": a.grain, "merge_min": 0xFFFFFFFF, "merge_ratio": 1}
     for sh in ([1, 1, 1], [64, 1, 1], [4096, 1, 1], [16, 16, 16], [64, 64, 1]):
         for _ in range(max(1, a.warmup)):
             hc.run_join(q, [ix] * 3, shares=sh, **knobs)
@@ -949,8 +963,10 @@ def kary_workload(a, world, rank, local):
     (tensor_relations), count mode, in the loop order hc_choose_korder picks;
     the step is one k-ary join over resident 3-level CoCo indexes (built
     once, timed separately).  Metric: results per second.  Roofline of the
-    search kernel: 4 bytes per unit of the work measure (sum over loops and
-    bindings of lists x shortest list) per launch.  A bounded sample
+    search kernel: the indexes' levels read once per launch, which it is far
+    from (issue of its intersections bounds it); beside it the rate by 4 bytes
+    per unit of the work measure (sum over loops and bindings of lists x
+    shortest list), which lists kept as bitmaps do not read.  A bounded sample
     (tensor_sample) is counted by the oracle and by the GPU on the same
     rows."""
     import numpy as np
@@ -1030,15 +1046,18 @@ def kary_workload(a, world, rank, local):
     peak, peak_kind = measured_hbm_peak()
     kms = kern_ms / a.steps
     metric = "LW results/s (count)" if a.workload == "lw" else "CT results/s (count)"
-    achieved = 4.0 * work / (kms / 1e3) / 1e9
+    level_bytes = 4 * sum(ix.v(d).shape[0] for ix in ixs for d in range(ix.arity))
+    achieved = level_bytes / (kms / 1e3) / 1e9
     # the committed capture covers LW over ST-Dense's [512]^3 cubes in one cell
     profiled = (a.workload == "lw" and a.lw_n == 512 and a.tensor == "dense" and kshares == (1, 1, 1, 1))
-    roofline = {"bound": "hbm", "kernel": "kjoin_kernel<4> (k-ary search)", "achieved": round(achieved, 1),
+    roofline = {"bound": "issue", "kernel": "kjoin_kernel<4> (k-ary search)", "achieved": round(achieved, 1),
                 "launches_per_step": 1,
                 "peak": peak, "peak_kind": peak_kind, "unit": "GB/s", "frac": round(achieved / peak, 4),
                 "traffic": profiled_traffic(KJOIN_PROFILE_NOTE, ("hc_kary.cu", "hc_internal.cuh")) if profiled else None,
-                "alg_bytes_per_launch": 4 * work, "avg_launch_ms": round(kms, 3),
-                "note": "work measure x 4 B; short lists are L1/L2-resident, so this can exceed what DRAM moves"}
+                "alg_bytes_per_launch": level_bytes, "avg_launch_ms": round(kms, 3),
+                "work_gbs": round(4.0 * work / (kms / 1e3) / 1e9, 1),
+                "note": "achieved: the indexes' levels read once; work_gbs: work measure x 4 B, most of which is read "
+                        "from L1/L2 or, for lists kept as bitmaps, at a bit a value"}
 
     e2e = None
     if not a.no_e2e:
