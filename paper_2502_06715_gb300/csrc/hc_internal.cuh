@@ -400,15 +400,18 @@ __device__ __forceinline__ bool dir_find(P a, const uint4* __restrict__ g, uint3
 }
 
 // ------------------------------------------------------------ dense bitmaps
-// Runs that hold about one in eight of the values they span, or more, are
-// also kept as bitmaps, at 8 bits a value of the level: a run a[lo, hi) of
+// k-ary levels whose average run fills a sixteenth of the level's value range
+// or more (build_kindex_impl) also keep as bitmaps those of their runs that
+// hold about one in eight of the values they span, or more, at 8 bits a value
+// of the level.  The first choice is per level: full runs of a level that is
+// wide as a whole (a block-diagonal tensor) get none.  A run a[lo, hi) of
 // n >= DIR_MIN values owns the 32-bit words that lie wholly in bytes [lo, hi)
 // of an array (so runs share no word), and is dense when its values fit
 // there: with vbase = vmin rounded down to a multiple of 32, bit b of its
 // word w stands for the value vbase + 32 w + b.  A dense run is searched by
 // one bit, and two of them intersect word by word.  The array starts with a
 // header of DENSE_HEAD words, the first of which is nonzero when any run is
-// dense (a large sparse graph has none, and its searches skip all this).
+// dense (the searches of a level without dense runs skip all this).
 constexpr uint32_t DENSE_HEAD = 4;
 
 struct Dense {

@@ -419,11 +419,11 @@ struct Entry {
 // candidate, and four candidates keep a round's lanes and its memory reads
 // busy; a unit of a deeper query carries a whole subtree of a hub or almost
 // nothing, so its items may be single units and more of them are wanted.
-// With 64 always, small and skewed graphs left most of the chip idle:
-// 4-cycle on R-MAT 10 / 13 14.5 / 39.7 -> 0.74 / 19.0 ms, 4-clique on R-MAT 12
-// 3.9 -> 0.75, triangle on 4,096 vertices and 32,768 edges 0.180 -> 0.101 a
-// call; the 4-clique on R-MAT 17 (40.3 -> 38.9) and the triangle on R-MAT 20
-// (7.81) are the upper end.
+// With 64 always, small and skewed graphs left most of the chip idle, in ms a
+// call: 4-cycle on R-MAT 10 / 13 14.0 / 38.1 -> 0.70 / 18.8, 4-clique on R-MAT
+// 12 3.5 -> 0.73, triangle on 4,096 vertices and 32,768 edges 0.167 -> 0.084.
+// The 4-clique on R-MAT 17 (42.4 -> 41.8) and the triangle on R-MAT 20 (7.85,
+// 7.84) are the upper end.
 __host__ __device__ inline uint32_t auto_grain(uint64_t units, uint64_t warps, int nlev) {
     const uint64_t per = nlev >= 4 ? 16 : 4, least = nlev >= 4 ? 1 : 4;
     const uint64_t g = units / (warps * per);
@@ -1402,9 +1402,10 @@ struct BQuery {
 };
 
 // One block: the batch's work units, from them each query's grain, and its
-// number of items.  A batch's queries end together, so twice as many items a
-// warp as a single query's are cut (96 graphs of about 30,000 edges: 13.9 ms
-// at 8 to 16 units an item, 14.5 at 32 and 16.0 at 64).
+// number of items: about 32 for each of `warps` (48 an SM), where a single
+// query's warps get 4 or, from 4 loops on, 16 (auto_grain), because a batch's
+// queries end together (96 graphs of about 30,000 edges: 13.9 ms at 8 to 16
+// units an item, 14.5 at 32 and 16.0 at 64).
 __global__ void __launch_bounds__(1024) batch_items_kernel(BQuery* __restrict__ qs, uint32_t n, uint64_t warps,
                                                            uint64_t* __restrict__ items) {
     __shared__ uint64_t s_sum[32];

@@ -479,8 +479,8 @@ __global__ void maxrun_kernel(const uint32_t* __restrict__ o1, uint64_t l1_max, 
 // consecutive positions.  Two threads find the runs that hold the tile's
 // first and last positions; the runs between them are marked at their starts
 // in shared memory, and a running maximum over the marks gives every position
-// its run (a binary search of the run starts per position cost more than the
-// rest of the kernel: 0.54 ms at 64 M rows, 0.46 ms so).  The value at position j
+// its run (0.47 ms at 64 M rows; 0.54 ms with a binary search of the run starts
+// per position).  The value at position j
 // opens the buckets above its predecessor's bucket up to its own and writes
 // entry (j, a[j], a[j+1], a[j+2]) for each (~0 past the run).  Buckets are
 // clamped to [0, nb - 1], so unsorted input (never produced by the builders
