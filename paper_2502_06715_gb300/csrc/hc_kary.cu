@@ -756,6 +756,11 @@ constexpr uint32_t KPAIR_MIN = 32;  // default per-binding threshold of the last
 constexpr uint32_t KP_BIT = 0x800u, KP_DIRECT = 0x200u, KP_DIR = 0x100u, KP_POS = 0x400u;
 constexpr uint32_t KDENSE_WORDS = 512;  // the word path of the last loop: words one lane takes, at most
 constexpr uint32_t KDENSE_TURN = 4;     // fixed cost of a parent whose words the warp shares, in words
+// What a search kernel is compiled for: counting, counting where the last
+// loop's lists may all be dense (kdense_last), writing tuples.  With the word
+// path in the one counting kernel, joins that have no use for it lost 7 to 9 %
+// to its registers (LW on sparse tensors of 8 M rows 0.93 -> 1.02 ms).
+enum KMode { KM_COUNT, KM_DENSE, KM_TUPLES };
 constexpr int KJ_MAXT = 128;      // threads per block of the search kernel, at most
 constexpr int KJ_WARPS = KJ_MAXT / 32;
 
@@ -786,7 +791,7 @@ struct KSrc {
 struct KPlan {
     int32_t nv, stats;
     uint32_t n_cells;
-    int32_t last_dense;  // every last-loop list's level has dense runs (set by the kernel)
+    int32_t last_dense;  // every last-loop list's level has dense runs (set by the kernel, KM_DENSE)
     uint32_t pair_min;  // last-loop parents with at least this many candidates take the per-binding path
     int32_t nsrc[HC_KMAX_VARS];
     int32_t var_of_loop[HC_KMAX_VARS];
@@ -1081,7 +1086,7 @@ __device__ __forceinline__ uint32_t kdense_count(const KDense& K, int ns, uint32
 // Start loop L with parents 0..nb-1: each parent's shortest list and the
 // prefix of their candidate counts.  Loop 1 has the entry as its only
 // parent and takes candidates [t0, t1) of its shortest list.
-template <int NV, bool MAT>
+template <int NV, KMode M>
 __device__ __forceinline__ void kinit_level(const KPlan& P, KWarp<NV>& S, int L, uint32_t nb, uint32_t t0,
                                             uint32_t t1, uint64_t& work, uint64_t& cnt) {
     const uint32_t lane = lane_id();
@@ -1116,7 +1121,7 @@ __device__ __forceinline__ void kinit_level(const KPlan& P, KWarp<NV>& S, int L,
     // longer than nb turns of 1/32 of it and KDENSE_TURN words (LW on a box of
     // 16 x 16 x 16 x 8000: 0.25 ms on lanes, 0.07 ms in turns)
     bool lng = false;
-    if (!MAT && L == NV - 1 && L > 1 && P.last_dense && lane < nb && c >= DIR_MIN) {
+    if (M == KM_DENSE && L == NV - 1 && L > 1 && P.last_dense && lane < nb && c >= DIR_MIN) {
         const uint32_t c32 = (uint32_t)c;
         KDense K;
         if ((c32 < P.pair_min || c32 <= nb * (c32 / 32 + 32 * KDENSE_TURN)) && kdense_init<NV>(P, S, lane, K) &&
@@ -1155,9 +1160,10 @@ __device__ __forceinline__ void kinit_level(const KPlan& P, KWarp<NV>& S, int L,
 // range, bounds and search kind (KP_*) are the same for every candidate, so
 // one lane per list sets them up once, in one shared-memory record.  The
 // last loop's lists are the atoms' last levels (no positions are needed).
-template <int NV, bool MAT>
+template <int NV, KMode M>
 __device__ __forceinline__ void kpair(const KPlan& P, KWarp<NV>& S, uint32_t b, uint64_t& cnt, JoinCtl* ctl,
                                       uint32_t* __restrict__ out, uint64_t cap) {
+    constexpr bool MAT = M == KM_TUPLES;
     constexpr int L = NV - 1, li = NV - 2;
     const uint32_t lane = lane_id();
     const uint32_t d = S.drv[li][b];
@@ -1168,7 +1174,7 @@ __device__ __forceinline__ void kpair(const KPlan& P, KWarp<NV>& S, uint32_t b, 
         if (lane == 0) cnt += a1 - a0;
         return;
     }
-    if (!MAT && P.last_dense) {  // all lists dense: the words of their AND, spread over the lanes
+    if (M == KM_DENSE && P.last_dense) {  // all lists dense: the words of their AND, spread over the lanes
         KDense K;
         if (kdense_init<NV>(P, S, b, K)) {
             cnt += kdense_count(K, ns, lane, 32);
@@ -1316,11 +1322,12 @@ __device__ __forceinline__ void kpair(const KPlan& P, KWarp<NV>& S, uint32_t b, 
 }
 
 // Walk loops 1..NV-1 below the entry in S, loop 1 over candidates [t0, t1).
-template <int NV, bool MAT>
+template <int NV, KMode M>
 __device__ void kwalk(const KPlan& P, KWarp<NV>& S, uint32_t t0, uint32_t t1, uint64_t& cnt, uint64_t& work,
                       JoinCtl* ctl, uint32_t* __restrict__ out, uint64_t cap) {
     const uint32_t lane = lane_id();
-    kinit_level<NV, MAT>(P, S, 1, 1, t0, t1, work, cnt);
+    constexpr bool MAT = M == KM_TUPLES;
+    kinit_level<NV, M>(P, S, 1, 1, t0, t1, work, cnt);
     int L = 1;
     while (true) {
         const int li = L - 1;
@@ -1333,7 +1340,7 @@ __device__ void kwalk(const KPlan& P, KWarp<NV>& S, uint32_t t0, uint32_t t1, ui
                 while (lm) {
                     const uint32_t b = __ffs(lm) - 1;
                     lm &= lm - 1;
-                    kpair<NV, MAT>(P, S, b, cnt, ctl, out, cap);
+                    kpair<NV, M>(P, S, b, cnt, ctl, out, cap);
                 }
             }
             if (L == 1) break;
@@ -1423,7 +1430,7 @@ __device__ void kwalk(const KPlan& P, KWarp<NV>& S, uint32_t t0, uint32_t t1, ui
         __syncwarp();
         if (m) {
             ++L;
-            kinit_level<NV, MAT>(P, S, L, (uint32_t)__popc(m), 0, 0, work, cnt);
+            kinit_level<NV, M>(P, S, L, (uint32_t)__popc(m), 0, 0, work, cnt);
         }
     }
 }
@@ -1431,12 +1438,13 @@ __device__ void kwalk(const KPlan& P, KWarp<NV>& S, uint32_t t0, uint32_t t1, ui
 // Persistent search kernel: warps take work items of `grain` loop-1
 // candidates (0: sized so that each warp gets about 8 items) from an atomic
 // counter, over the concatenation of all entries' candidates.
-template <int NV, bool MAT>
+template <int NV, KMode M>
 __global__ void __launch_bounds__(KJ_MAXT) kjoin_kernel(const KPlan* __restrict__ gP,
                                                         const KEntry* __restrict__ entries,
                                                         const uint64_t* __restrict__ unit_off, JoinCtl* ctl,
                                                         uint32_t grain_in, uint32_t* __restrict__ out, uint64_t cap,
                                                         uint64_t* __restrict__ cell_counts) {
+    constexpr bool MAT = M == KM_TUPLES;
     __shared__ KPlan P;
     __shared__ KWarp<NV> WS[KJ_WARPS];
     load_kplan(P, gP);
@@ -1444,13 +1452,13 @@ __global__ void __launch_bounds__(KJ_MAXT) kjoin_kernel(const KPlan* __restrict_
     KWarp<NV>& S = WS[w];
     if (dev_err_set(&ctl->err)) return;  // the unit-offset scan gave up a wait
     if (threadIdx.x == 0) {  // levels without dense runs: their bitmaps are not looked at
-        int all = P.nsrc[NV - 1] > 1;  // a single list has nothing to intersect
+        int all = 1;
         for (int q = 0; q < P.nsrc[NV - 1]; ++q) {
             KSrc& s = P.src[NV - 1][q];
             if (s.b != nullptr && __ldg(s.b) == 0) s.b = nullptr;
             all &= s.b != nullptr;
         }
-        P.last_dense = all;
+        if (M == KM_DENSE) P.last_dense = all;
     }
     __syncthreads();
     const uint32_t ne = ctl->n_entries;
@@ -1500,7 +1508,7 @@ __global__ void __launch_bounds__(KJ_MAXT) kjoin_kernel(const KPlan* __restrict_
                 __syncwarp();
                 const uint64_t u_end = u1 < ee ? u1 : ee;
                 if (!MAT && cell_counts) S.c0[lane] = cnt;
-                kwalk<NV, MAT>(P, S, (uint32_t)(u0 - eb), (uint32_t)(u_end - eb), cnt, work, ctl, out, cap);
+                kwalk<NV, M>(P, S, (uint32_t)(u0 - eb), (uint32_t)(u_end - eb), cnt, work, ctl, out, cap);
                 if (!MAT && cell_counts) {
                     const uint64_t dc = warp_sum64(cnt - S.c0[lane]);
                     if (lane == 0 && dc)
@@ -1521,26 +1529,26 @@ __global__ void __launch_bounds__(KJ_MAXT) kjoin_kernel(const KPlan* __restrict_
     }
 }
 
-template <int NV, bool MAT>
+template <int NV, KMode M>
 hc_status launch_kjoin_t(int threads, const KPlan* P, const KEntry* entries, const uint64_t* unit_off, JoinCtl* ctl,
                          uint32_t grain, uint32_t* out, uint64_t cap, uint64_t* cell_counts, cudaStream_t s) {
     int per_sm = 0;
-    HC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kjoin_kernel<NV, MAT>, threads, 0));
+    HC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kjoin_kernel<NV, M>, threads, 0));
     const int grid = num_sms() * std::max(1, per_sm);
-    kjoin_kernel<NV, MAT><<<grid, threads, 0, s>>>(P, entries, unit_off, ctl, grain, out, cap, cell_counts);
+    kjoin_kernel<NV, M><<<grid, threads, 0, s>>>(P, entries, unit_off, ctl, grain, out, cap, cell_counts);
     HC_CUDA_TRY(launch_check());
     return HC_OK;
 }
 
-template <bool MAT>
+template <KMode M>
 hc_status launch_kjoin(int nv, int threads, const KPlan* P, const KEntry* entries, const uint64_t* unit_off,
                        JoinCtl* ctl, uint32_t grain, uint32_t* out, uint64_t cap, uint64_t* cc, cudaStream_t s) {
     switch (nv) {
-        case 2: return launch_kjoin_t<2, MAT>(threads, P, entries, unit_off, ctl, grain, out, cap, cc, s);
-        case 3: return launch_kjoin_t<3, MAT>(threads, P, entries, unit_off, ctl, grain, out, cap, cc, s);
-        case 4: return launch_kjoin_t<4, MAT>(threads, P, entries, unit_off, ctl, grain, out, cap, cc, s);
-        case 5: return launch_kjoin_t<5, MAT>(threads, P, entries, unit_off, ctl, grain, out, cap, cc, s);
-        case 6: return launch_kjoin_t<6, MAT>(threads, P, entries, unit_off, ctl, grain, out, cap, cc, s);
+        case 2: return launch_kjoin_t<2, M == KM_DENSE ? KM_COUNT : M>(threads, P, entries, unit_off, ctl, grain, out, cap, cc, s);
+        case 3: return launch_kjoin_t<3, M>(threads, P, entries, unit_off, ctl, grain, out, cap, cc, s);
+        case 4: return launch_kjoin_t<4, M>(threads, P, entries, unit_off, ctl, grain, out, cap, cc, s);
+        case 5: return launch_kjoin_t<5, M>(threads, P, entries, unit_off, ctl, grain, out, cap, cc, s);
+        case 6: return launch_kjoin_t<6, M>(threads, P, entries, unit_off, ctl, grain, out, cap, cc, s);
         default: return fail(HC_ERR_CAPACITY, "run_kjoin: unsupported number of variables");
     }
 }
@@ -1550,6 +1558,15 @@ hc_status read_kctl(hc_result* R) {
     HC_CUDA_TRY(cudaStreamSynchronize(R->stream));
     if (R->h_ctl.err & DEV_ERR_TIMEOUT) return fail(HC_ERR_TIMEOUT, "run_kjoin: a bounded device wait gave up");
     return HC_OK;
+}
+
+// Whether the word path can serve the last loop: two lists or more, below a
+// loop that binds their parents, each of a level that keeps bitmaps.
+bool kdense_last(const KPlan& P) {
+    const int L = P.nv - 1;
+    bool all = L > 1 && P.nsrc[L] > 1;
+    for (int q = 0; all && q < P.nsrc[L]; ++q) all = P.src[L][q].b != nullptr;
+    return all;
 }
 
 // Validation and the lists of every loop (host only).
@@ -1747,11 +1764,11 @@ hc_status run_kjoin_impl(const hc_kquery* q, const hc_kindex* const* idx, const 
                                                              0, cc);
             HC_CUDA_TRY(launch_check());
         } else if (mat) {
-            HC_TRY(launch_kjoin<true>((int)nv, threads, dP, entries, unit_off, ctl, dp.item_grain, tup, cap, nullptr,
+            HC_TRY(launch_kjoin<KM_TUPLES>((int)nv, threads, dP, entries, unit_off, ctl, dp.item_grain, tup, cap, nullptr,
                                       s));
         } else {
-            HC_TRY(
-                launch_kjoin<false>((int)nv, threads, dP, entries, unit_off, ctl, dp.item_grain, nullptr, 0, cc, s));
+            auto* launch = kdense_last(P) ? launch_kjoin<KM_DENSE> : launch_kjoin<KM_COUNT>;
+            HC_TRY(launch((int)nv, threads, dP, entries, unit_off, ctl, dp.item_grain, nullptr, 0, cc, s));
         }
         if (timed) HC_TRY(time_mark(R, true, s));
         R->n_search++;
