@@ -302,7 +302,8 @@ typedef struct {
     uint32_t merge_ratio;         /* ... and within this length ratio are intersected    */
                                   /* by a warp block merge, others by binary search      */
                                   /* (0: 32 and 4; 0xFFFFFFFF: never merge; with both 0   */
-                                  /* only where the longer list has no directory)        */
+                                  /* only where the longer list has no directory; in a   */
+                                  /* batch, only queries of few rows)                    */
     uint32_t slice_grain;         /* 4+ loops: loop-3 candidates per work slice of a     */
                                   /* loop-2 binding (0: default 256; 0xFFFFFFFF: none)   */
     uint32_t lift_arena;          /* query rewriting: words of device scratch per warp   */

@@ -464,8 +464,10 @@ struct Acc {
     uint32_t* obuf;   // the warp's staging buffer of OBUF values (materialize), or NULL
     uint64_t* cprof;  // per-cell profile [cells][2] (work units, SM cycles), or NULL
 };
-// A batched query's: its lists merge whichever is longer (batch_create).
+// A batched query's: its lists merge whichever is longer, or never (batch_create).
 struct BatchAcc : Acc {};
+constexpr uint64_t BATCH_MERGE_ROWS = 1u << 15;       // rows from which a batched query's lists are not merged,
+constexpr uint64_t BATCH_MERGE_ROWS_DEEP = 1u << 12;  // and from 4 loops on
 
 // Output slot of the lane holding rank r among the k = popc(ball) matches
 // of this round (all lanes call).  Two-pass mode: consecutive slots from
@@ -1395,18 +1397,37 @@ struct BQuery {
     const uint32_t *e_cell, *e_x, *e_rng, *e_split;
     const uint64_t* uoff;
     JoinCtl* ctl;
-    uint32_t grain;  // as asked for (0: auto_grain over the batch's units)
+    uint32_t grain;  // as asked for (0: batch_grain)
     uint32_t run;    // the grain of this launch (batch_items_kernel)
     uint32_t nlev;
     uint32_t shape;  // 0: the kernel's first shape, 1: its second (all-shapes kernel: the shape class)
 };
 
+// Work units per item of a batched query that names none, from the units of
+// the whole batch.  An item costs a search of its query, entry and ranges, so
+// a batch wants longer ones than a query alone: two for each resident warp are
+// enough, up to a length past which the last ones are waited for.  That length
+// is shorter where queries of 3 loops and of more share the launch (`mixed`),
+// and for the deeper ones, whose units are subtrees, but for those not below
+// 1/24 of a warp's share.  ms a launch at 4 / 8 / 16 / 32 / 64 units: 300
+// triangles of 3,000 edges 0.34 / 0.24 / 0.20 / 0.20 / 0.21, 64 of 100,000 4.1 /
+// 2.6 / 2.0 / 1.7 / 1.6; 200 4-cliques of 3,000 1.05 / 0.90 / 0.85 / 0.88 / 1.00, 64
+// of 100,000 45.7 / 40.9 / 37.7 / 36.0 / 36.4.  Of both, at 2 / 4 / 8 / 16 / 24 units
+// for the 4-cliques: 40 of 15,000 2.35 / 2.17 / 2.33 / 2.60 / 2.82, 96 of 5,000
+// 1.71 / 1.64 / 1.56 / 1.72 / 1.72, 96 of 30,000 15.3 / 13.5 / 12.6 / 12.5 / 12.9,
+// 96 of 60,000 35.6 / 31.1 / 28.7 / 27.7 / 27.5 (28.9 at 33).  Cutting 32 items a
+// warp whatever the shapes took 0.34, 1.8, 1.7 and 39.2 ms, and 2.3, 1.9, 13.0.
+__device__ __forceinline__ uint32_t batch_grain(uint64_t units, uint32_t sms, uint32_t nlev, bool mixed) {
+    const uint64_t warps = (uint64_t)sms * (nlev >= 4 ? 48 : 64);
+    const uint64_t share = units / (2 * warps);
+    if (nlev < 4) return (uint32_t)max((uint64_t)4, min(share, (uint64_t)(mixed ? 16 : 64)));
+    const uint64_t most = max((uint64_t)(mixed ? 4 : 16), min((uint64_t)(mixed ? 24 : 64), units / (24 * warps)));
+    return (uint32_t)max((uint64_t)1, min(share, most));
+}
+
 // One block: the batch's work units, from them each query's grain, and its
-// number of items: about 32 for each of `warps` (48 an SM), where a single
-// query's warps get 4 or, from 4 loops on, 16 (auto_grain), because a batch's
-// queries end together (96 graphs of about 30,000 edges: 13.9 ms at 8 to 16
-// units an item, 14.5 at 32 and 16.0 at 64).
-__global__ void __launch_bounds__(1024) batch_items_kernel(BQuery* __restrict__ qs, uint32_t n, uint64_t warps,
+// number of items.
+__global__ void __launch_bounds__(1024) batch_items_kernel(BQuery* __restrict__ qs, uint32_t n, uint32_t sms, bool mixed,
                                                            uint64_t* __restrict__ items) {
     __shared__ uint64_t s_sum[32];
     uint64_t sum = 0;
@@ -1421,7 +1442,7 @@ __global__ void __launch_bounds__(1024) batch_items_kernel(BQuery* __restrict__ 
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
         BQuery& b = qs[i];
         const uint64_t U = units(b);
-        b.run = b.grain ? b.grain : auto_grain(total / 2, b.nlev >= 4 ? warps : 4 * warps, (int)b.nlev);
+        b.run = b.grain ? b.grain : batch_grain(total, sms, b.nlev, mixed);
         items[i] = (U + b.run - 1) / b.run;
     }
 }
@@ -2581,6 +2602,7 @@ struct hc_batch {
     uint32_t l0_tiles = 0;         // loop-1 tiles of all queries
     int class_a = 0, class_b = 0;
     bool all_shapes = false;  // more than two shape classes: gj_batch_all_kernel
+    bool mixed = false;       // queries of 3 loops and of more
     uint32_t* d_arena = nullptr;  // lifted lists (query rewriting), arena_stride words per warp
     uint32_t arena_stride = 0;
     cudaGraph_t graph = nullptr;
@@ -2622,11 +2644,21 @@ hc_status batch_create(const hc_query* qs, const hc_index* const* idx_flat, cons
         if (prm[i].mode != HC_MODE_COUNT) return bail(fail(HC_ERR_ARG, "batch: queries run in count mode"));
         hc_status st = plan_query(&qs[i], idx_flat + off, &prm[i], s, &B->plans[i]);
         if (st != HC_OK) return bail(st);
-        // the batched kernels, at 40 registers for two shapes, search slower
-        // than they merge, so the automatic rule is not theirs: five kinds of
-        // batch, 24 to 96 queries of 1,500 to 60,000 edges, take as long or up
-        // to 5 % longer with it (96 of 30,000: 13.57 against 13.07 ms)
-        B->plans[i].P.merge_min = prm[i].merge_min ? prm[i].merge_min : 32;
+        // by default a batch merges a small query's lists whichever is longer,
+        // and searches all of a large one's: triangles of 14,000 rows 0.315 ms
+        // merged and 0.331 searched, of 79,000 1.62 and 1.59, of 390,000 3.89 and
+        // 3.62; 4-cliques of 1,600 rows 0.850 and 0.855, of 14,000 3.67 and 3.68, of
+        // 79,000 38.9 and 36.0; among triangles, 96 of 30,000 rows 13.2 ms when the
+        // 4-cliques are searched from 32,768 rows on, 12.4 from 4,096
+        {
+            DPlan& P = B->plans[i].P;
+            uint64_t rows = 0;
+            for (uint32_t j = 0; j < qs[i].n_atoms; ++j) rows = std::max(rows, idx_flat[off + j]->n);
+            const bool by_size = prm[i].merge_min == 0 && prm[i].merge_ratio == 0 && P.dir_min == DIR_MIN;
+            const bool searched = by_size && rows >= (P.nlev >= 4 ? BATCH_MERGE_ROWS_DEEP : BATCH_MERGE_ROWS);
+            P.merge_min = searched ? 0xFFFFFFFFu : prm[i].merge_min ? prm[i].merge_min : 32;
+            B->mixed = B->mixed || (B->plans[i].nv >= 4) != (B->plans[0].nv >= 4);
+        }
         if (B->plans[i].P.lift) B->arena_stride = std::max(B->arena_stride, B->plans[i].P.arena_words);
         off += qs[i].n_atoms;
         const int c = shape_class(B->plans[i]);
@@ -2702,7 +2734,7 @@ static hc_status batch_enqueue(hc_batch* B, cudaStream_t s) {
     l0_batch_kernel<<<std::min<unsigned>(B->l0_tiles, (unsigned)num_sms() * 6), L0_TILE, 0, s>>>(
         B->d_jobs, B->n, B->l0_tiles, B->d_ctr + 1, wait_limit_ns());
     HC_CUDA_TRY(launch_check());
-    batch_items_kernel<<<1, 1024, 0, s>>>(B->d_q, B->n, (uint64_t)num_sms() * 48, B->d_items);
+    batch_items_kernel<<<1, 1024, 0, s>>>(B->d_q, B->n, (uint32_t)num_sms(), B->mixed, B->d_items);
     HC_CUDA_TRY(launch_check());
     HC_TRY(exclusive_scan_u64(B->d_items, B->d_item_off, B->n, nullptr, &B->d_ctl[0].err, s));
     if (B->all_shapes) {
