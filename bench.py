@@ -597,8 +597,7 @@ def other_workload(a, world, rank, local):
     tune_s = time.perf_counter() - t
     sep_counts = [hc.run_join(q, l, **o).count for q, l, o in zip(qs, idx, opts)]
     side = torch.cuda.Stream(dev)
-    # a batch cuts its items over all its queries and merges by its own rule
-    b = hc.Batch(qs, idx, [{k: o[k] for k in ("shares", "slice_grain")} for o in opts], stream=side)
+    b = hc.Batch(qs, idx, opts, stream=side)
     l0 = hc.kernel_launches()
     b.capture(side)
     per_replay = hc.kernel_launches() - l0  # kernels recorded in the graph
@@ -964,7 +963,7 @@ def kary_workload(a, world, rank, local):
     the step is one k-ary join over resident 3-level CoCo indexes (built
     once, timed separately).  Metric: results per second.  Roofline of the
     search kernel: the indexes' levels read once per launch, which it is far
-    from (issue of its intersections bounds it); beside it the rate by 4 bytes
+    from (its loads through L1 bound it); beside it the rate by 4 bytes
     per unit of the work measure (sum over loops and bindings of lists x
     shortest list), which lists kept as bitmaps do not read.  A bounded sample
     (tensor_sample) is counted by the oracle and by the GPU on the same
@@ -1050,7 +1049,7 @@ def kary_workload(a, world, rank, local):
     achieved = level_bytes / (kms / 1e3) / 1e9
     # the committed capture covers LW over ST-Dense's [512]^3 cubes in one cell
     profiled = (a.workload == "lw" and a.lw_n == 512 and a.tensor == "dense" and kshares == (1, 1, 1, 1))
-    roofline = {"bound": "issue", "kernel": "kjoin_kernel<4> (k-ary search)", "achieved": round(achieved, 1),
+    roofline = {"bound": "l1", "kernel": "kjoin_kernel<4> (k-ary search)", "achieved": round(achieved, 1),
                 "launches_per_step": 1,
                 "peak": peak, "peak_kind": peak_kind, "unit": "GB/s", "frac": round(achieved / peak, 4),
                 "traffic": profiled_traffic(KJOIN_PROFILE_NOTE, ("hc_kary.cu", "hc_internal.cuh")) if profiled else None,
