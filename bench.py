@@ -246,7 +246,8 @@ def schedule_name(shares, item_grain, merge_min, merge_ratio) -> str:
 def profiled_traffic(note: str = None, sources=("hc_join.cu", "hc_internal.cuh"), schedule: str = None):
     """Per-launch DRAM bytes of a kernel from a committed ncu summary, if it
     was taken on the current source of the files that hold the kernel and,
-    where the bytes depend on it, under the same cells and schedule."""
+    where the bytes depend on it, under the same cells and schedule (a note
+    names each schedule that makes the captured launch)."""
     try:
         text = open(note or PROFILE_NOTE).read()
     except OSError:
@@ -258,8 +259,7 @@ def profiled_traffic(note: str = None, sources=("hc_join.cu", "hc_internal.cuh")
     if source_hash(sources) != h.group(1):
         return None
     if schedule is not None:
-        taken = re.search(r"^\s*schedule: (.+?)\s*$", text, re.M)
-        if not taken or taken.group(1) != schedule:
+        if schedule not in re.findall(r"^\s*schedule: (.+?)\s*$", text, re.M):
             return None
     return int(m.group(1))
 

@@ -16,8 +16,8 @@ OFF = 0xFFFFFFFF
 def _note(tmp_path, schedule):
     sources = ("hc_join.cu", "hc_internal.cuh")
     text = f"    traffic_bytes_per_launch: 123456\n    source_sha256: {bench.source_hash(sources)}\n"
-    if schedule is not None:
-        text += f"    schedule: {schedule}\n"
+    for s in [schedule] if isinstance(schedule, str) else schedule or []:
+        text += f"    schedule: {s}\n"
     path = tmp_path / "note.md"
     path.write_text(text)
     return str(path)
@@ -33,4 +33,7 @@ def test_traffic_belongs_to_the_schedule(tmp_path, args, name):
     other = bench.schedule_name(args[0], 256, *args[2:])
     assert bench.profiled_traffic(note, schedule=other) is None
     assert bench.profiled_traffic(_note(tmp_path, None), schedule=name) is None
+    both = _note(tmp_path, [other, name])  # two names of one launch
+    assert bench.profiled_traffic(both, schedule=name) == bench.profiled_traffic(both, schedule=other) == 123456
+    note = _note(tmp_path, name)
     assert bench.profiled_traffic(note) == 123456  # a kernel with one schedule names none
