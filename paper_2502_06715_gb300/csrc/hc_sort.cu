@@ -697,12 +697,31 @@ int grid_for(uint64_t n, int threads, int per_sm) {
 struct Tmp {
     cudaStream_t s;
     std::vector<void*> ptrs;
+    char* block = nullptr;  // reserved ahead, not yet handed out
+    size_t left = 0;
     explicit Tmp(cudaStream_t st) : s(st) {}
+    static size_t whole(size_t bytes) { return (bytes + 255) / 256 * 256; }
+    // One block for what later get() calls ask for; without the room for it
+    // they allocate one by one.
+    void reserve(size_t bytes) {
+        void* v = nullptr;
+        if (dev_alloc(&v, bytes, s) != HC_OK) return;
+        ptrs.push_back(v);
+        block = (char*)v;
+        left = bytes;
+    }
     ~Tmp() {
         for (void* p : ptrs) dev_free(p, s);
     }
     template <typename T>
     hc_status get(T** p, size_t count) {
+        const size_t need = whole(std::max<size_t>(count, 1) * sizeof(T));
+        if (need <= left) {
+            *p = (T*)block;
+            block += need;
+            left -= need;
+            return HC_OK;
+        }
         void* v = nullptr;
         HC_TRY(dev_alloc(&v, std::max<size_t>(count, 1) * sizeof(T), s));
         ptrs.push_back(v);
@@ -830,14 +849,18 @@ std::vector<DigitSpec> key_digits(uint32_t max_first, uint32_t max_second) {
 
 }  // namespace
 
+// A directory whose memory *out_g already holds is built there.
 hc_status build_directory(const uint32_t* a, uint64_t alen, const uint32_t* o, uint64_t nruns_max,
                           const uint32_t* d_nruns, const uint32_t* d_err, cudaStream_t s, uint4** out_g,
                           uint32_t** out_b) {
+    void* p = *out_g;
     *out_g = nullptr;
     if (out_b) *out_b = nullptr;
-    if (alen < DIR_MIN || nruns_max == 0) return HC_OK;  // no run can have a directory
-    void* p = nullptr;
-    HC_TRY(dev_alloc(&p, alen * sizeof(uint4), s));
+    if (alen < DIR_MIN || nruns_max == 0) {  // no run can have a directory
+        dev_free(p, s);
+        return HC_OK;
+    }
+    if (!p) HC_TRY(dev_alloc(&p, alen * sizeof(uint4), s));
     void* bp = nullptr;
     if (out_b) {
         const size_t bbytes = (alen + 3) / 4 * 4 + DENSE_HEAD * 4;  // 8 bits a value, whole words, and the header
@@ -872,9 +895,7 @@ hc_status build_level_directories(hc_index* idx, cudaStream_t s);
 // The keys and the levels V1, O1 and V2 of n rows, in one block that d_keys
 // owns, each from a 256-byte boundary.  Freed and taken one by one they broke
 // up the pool's free space, and cudaMallocAsync then unmapped and mapped
-// memory to find room: 0.06 to 0.65 ms of a build of 64 M rows, by what the
-// process ran before (4.20 ms on its own and after a batch, 3.90 after other
-// joins; 3.84, 3.85 and 3.97 so).
+// memory to find room.
 template <class Index>
 static hc_status alloc_levels(Index* x, uint64_t n, cudaStream_t s) {
     const auto whole = [](uint64_t bytes) { return (bytes + 255) / 256 * 256; };
@@ -914,11 +935,27 @@ hc_status build_index_impl(const uint32_t* d_pairs, uint64_t n, uint32_t ao, uin
     void* p;
     if (alloc_levels(idx, n, s) != HC_OK) return bail(HC_ERR_OOM);
 
+    // All large blocks are taken here, ahead of the work and of the wait for
+    // the maxima: the levels, the directory's memory and the scratch.  In a
+    // pool that other streams have used, one that is asked for after a wait
+    // costs 50 us more, and block by block a build of 64 M rows spent 0.06 to
+    // 0.65 ms on them, by what the process ran before (4.20 ms on its own, 4.21
+    // after a batch, 3.90 after a burst of requests; 3.84, 3.85 and 3.91 so, and
+    // 1.9 M rows 300, 313 and 373 us; 296, 301 and 372).
+    if (n >= DIR_MIN && dev_alloc(&p, n * sizeof(uint4), s) == HC_OK) idx->d_g2 = (uint4*)p;
+
     hc_status st;
     LaunchTimer t_radix, t_boundary;
     t_radix.on = t_boundary.on = (flags & HC_BUILD_TIME_KERNELS) != 0;
     {
         Tmp tmp(s);
+        if (n > 0) {
+            const size_t pass_words = (n + PASS_TILE - 1) / PASS_TILE * RADIX;
+            const size_t scan_words = (n + SORT_TILE - 1) / SORT_TILE;
+            tmp.reserve(Tmp::whole(n * 8) + Tmp::whole(pass_words * 8) + Tmp::whole(scan_words * 8) +
+                        Tmp::whole(MAX_PASSES * RADIX * 4) + Tmp::whole(MAX_PASSES * sizeof(DigitSpec)) +
+                        Tmp::whole(sizeof(Ctl)));
+        }
         Ctl* d_ctl;
         if ((st = tmp.get(&d_ctl, 1)) != HC_OK) return bail(st);
         if (cudaMemsetAsync(d_ctl, 0, sizeof(Ctl), s) != cudaSuccess)
@@ -1009,8 +1046,12 @@ hc_status sort_pairs(const uint2* d_pairs, uint64_t n, uint32_t max_first, uint3
 // Directories of a built index: V2 by the runs of O1, and V1 as one run
 // when it has no position map.
 hc_status build_level_directories(hc_index* idx, cudaStream_t s) {
-    if (idx->max_run >= DIR_MIN)
+    if (idx->max_run >= DIR_MIN) {
         HC_TRY(build_directory(idx->d_v2, idx->n, idx->d_o1, idx->l1, nullptr, nullptr, s, &idx->d_g2, nullptr));
+    } else {  // no use for the memory taken ahead
+        dev_free(idx->d_g2, s);
+        idx->d_g2 = nullptr;
+    }
     if (idx->d_v1pos == nullptr && idx->l1 >= DIR_MIN)
         HC_TRY(build_directory(idx->d_v1, idx->l1, nullptr, idx->l1, nullptr, nullptr, s, &idx->d_g1, nullptr));
     return HC_OK;
