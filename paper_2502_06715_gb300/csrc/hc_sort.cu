@@ -697,31 +697,12 @@ int grid_for(uint64_t n, int threads, int per_sm) {
 struct Tmp {
     cudaStream_t s;
     std::vector<void*> ptrs;
-    char* block = nullptr;  // reserved ahead, not yet handed out
-    size_t left = 0;
     explicit Tmp(cudaStream_t st) : s(st) {}
-    static size_t whole(size_t bytes) { return (bytes + 255) / 256 * 256; }
-    // One block for what later get() calls ask for; without the room for it
-    // they allocate one by one.
-    void reserve(size_t bytes) {
-        void* v = nullptr;
-        if (dev_alloc(&v, bytes, s) != HC_OK) return;
-        ptrs.push_back(v);
-        block = (char*)v;
-        left = bytes;
-    }
     ~Tmp() {
         for (void* p : ptrs) dev_free(p, s);
     }
     template <typename T>
     hc_status get(T** p, size_t count) {
-        const size_t need = whole(std::max<size_t>(count, 1) * sizeof(T));
-        if (need <= left) {
-            *p = (T*)block;
-            block += need;
-            left -= need;
-            return HC_OK;
-        }
         void* v = nullptr;
         HC_TRY(dev_alloc(&v, std::max<size_t>(count, 1) * sizeof(T), s));
         ptrs.push_back(v);
@@ -935,13 +916,13 @@ hc_status build_index_impl(const uint32_t* d_pairs, uint64_t n, uint32_t ao, uin
     void* p;
     if (alloc_levels(idx, n, s) != HC_OK) return bail(HC_ERR_OOM);
 
-    // All large blocks are taken here, ahead of the work and of the wait for
-    // the maxima: the levels, the directory's memory and the scratch.  In a
-    // pool that other streams have used, one that is asked for after a wait
-    // costs 50 us more, and block by block a build of 64 M rows spent 0.06 to
-    // 0.65 ms on them, by what the process ran before (4.20 ms on its own, 4.21
-    // after a batch, 3.90 after a burst of requests; 3.84, 3.85 and 3.91 so, and
-    // 1.9 M rows 300, 313 and 373 us; 296, 301 and 372).
+    // The directory's memory too is taken here, ahead of the work and of the
+    // wait for the maxima: in a pool that other streams have used, a block that
+    // is asked for after a wait costs 50 us more.  Block by block a build of 64 M
+    // rows spent 0.06 to 0.65 ms on them, by what the process ran before (4.20 ms
+    // on its own, 4.21 after a batch, 3.90 after a burst of requests; 3.84, 3.85
+    // and 3.93 so, and 1.9 M rows 300, 313 and 373 us; 296, 303 and 375).  Without
+    // the room for it now it is asked for when it is built.
     if (n >= DIR_MIN && dev_alloc(&p, n * sizeof(uint4), s) == HC_OK) idx->d_g2 = (uint4*)p;
 
     hc_status st;
@@ -949,13 +930,6 @@ hc_status build_index_impl(const uint32_t* d_pairs, uint64_t n, uint32_t ao, uin
     t_radix.on = t_boundary.on = (flags & HC_BUILD_TIME_KERNELS) != 0;
     {
         Tmp tmp(s);
-        if (n > 0) {
-            const size_t pass_words = (n + PASS_TILE - 1) / PASS_TILE * RADIX;
-            const size_t scan_words = (n + SORT_TILE - 1) / SORT_TILE;
-            tmp.reserve(Tmp::whole(n * 8) + Tmp::whole(pass_words * 8) + Tmp::whole(scan_words * 8) +
-                        Tmp::whole(MAX_PASSES * RADIX * 4) + Tmp::whole(MAX_PASSES * sizeof(DigitSpec)) +
-                        Tmp::whole(sizeof(Ctl)));
-        }
         Ctl* d_ctl;
         if ((st = tmp.get(&d_ctl, 1)) != HC_OK) return bail(st);
         if (cudaMemsetAsync(d_ctl, 0, sizeof(Ctl), s) != cudaSuccess)

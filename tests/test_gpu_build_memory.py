@@ -1,7 +1,7 @@
 """The device memory a build holds at its peak and keeps.
 
-A build asks for its large blocks ahead: 20 bytes a row of keys and levels, 16
-of directory and, until it is done, about 8.4 of scratch.  An index without a
+A build holds 20 bytes a row of keys and levels, 16 of directory, asked for
+ahead, and, until it is done, about 8.4 of scratch.  An index without a
 run of 16 values or more gives the directory's block back.  Read from the
 device's default memory pool through the driver."""
 import ctypes
